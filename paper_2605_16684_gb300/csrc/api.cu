@@ -181,6 +181,7 @@ EsdgVolArgs vol_args(es_dg_t* h, const double* q_in, double* rhs_out) {
   a.rhs = rhs_out;
   a.vgeo = h->mixed ? (const void*)h->vgeo32 : (const void*)h->vgeo;
   a.vgeo64 = h->vgeo;
+  a.Ja = h->Ja;
   a.fflux = h->fflux;
   a.x = h->x;
   a.bg = (h->mixed && h->has_bg) ? h->bg3 : nullptr;
@@ -495,7 +496,7 @@ int create_impl(const es_dg_mesh* mesh, int N, es_dg_precision precision,
   if (!st) st = dev_alloc(h, (void**)&h->x, E * 3 * np * sizeof(double));
   if (!st) st = dev_alloc(h, (void**)&h->J, E * np * sizeof(double));
   if (!st) st = dev_alloc(h, (void**)&h->Ja, E * 9 * np * sizeof(double));
-  if (!st) st = dev_alloc(h, (void**)&h->vgeo, E * ESDG_NVGEO * np * sizeof(double));
+  if (!st) st = dev_alloc(h, (void**)&h->vgeo, ESDG_VGEO_BYTES(E, np));
   if (!st) st = dev_alloc(h, (void**)&h->vgeo32, E * ESDG_NVGEO * np * sizeof(float));
   if (!st) st = dev_alloc(h, (void**)&h->fgeo, (size_t)g.nfaces * 5 * nf2 * sizeof(double));
   if (!st)
@@ -521,7 +522,7 @@ int create_impl(const es_dg_mesh* mesh, int N, es_dg_precision precision,
           {h->x, o->x, E * 3 * np * sizeof(double)},
           {h->J, o->J, E * np * sizeof(double)},
           {h->Ja, o->Ja, E * 9 * np * sizeof(double)},
-          {h->vgeo, o->vgeo, E * ESDG_NVGEO * np * sizeof(double)},
+          {h->vgeo, o->vgeo, ESDG_VGEO_BYTES(E, np)},
           {h->vgeo32, o->vgeo32, E * ESDG_NVGEO * np * sizeof(float)},
           {h->fgeo, o->fgeo, nfg * sizeof(double)}};
       for (int k = 0; k < 6 && e == cudaSuccess; k++)

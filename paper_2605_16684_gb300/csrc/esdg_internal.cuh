@@ -2,8 +2,9 @@
 //
 // Data layout in HBM (one handle, E elements, np = Nq^3 nodes each):
 //   q, dq, rhs      double [E][5][np]            element-major, variable, node
-//   vgeo            double [E][11][np]           1/2 Ja^d_c (9), 1/J, phi
-//   vgeo32          float  [E][11][np]           same, FP32 copy (mixed mode)
+//   vgeo            double [E][11][np]           1/2 Ja^d_c (9, fixed-point limbs), 1/J, phi;
+//                                                then int [E], the limbs' scales (volume_fx.cuh)
+//   vgeo32          float  [E][11][np]           the same in FP32 (mixed mode)
 //   x               double [E][3][np]            node coordinates
 //   fgeo            double [F][5][Nq^2]          nhat (3), s / w_end, phi per face node
 //   fflux           double/float [F][5][Nq^2]    (s / w_end) F* per face node
@@ -17,6 +18,8 @@
 #define ESDG_NV 5
 #define ESDG_MAXNQ 8
 #define ESDG_NVGEO 11
+// bytes of vgeo
+#define ESDG_VGEO_BYTES(E, np) ((E) * ESDG_NVGEO * (np) * sizeof(double) + (E) * sizeof(int))
 
 struct EsdgLGL {  // LGL operators, passed by value (lives in the constant bank)
   int N;
@@ -27,6 +30,12 @@ struct EsdgLGL {  // LGL operators, passed by value (lives in the constant bank)
   float Dtf[ESDG_MAXNQ][ESDG_MAXNQ];  // FP32 copy for the mixed-precision pair loop
   double xi_lo[ESDG_MAXNQ];           // low parts (xi = xi + xi_lo, D = D + D_lo) for the
   double D_lo[ESDG_MAXNQ][ESDG_MAXNQ];  // double-double geometry construction
+  // fixed-point tables of the FP64 pair pass (limbs h 2^30 + l, volume_fx.cuh):
+  // Q_il = w_i Dt_il times 2^59, 1/w_i times 2^(60 - wm), w_0 times 2^(59 + wm)
+  int Qh[ESDG_MAXNQ][ESDG_MAXNQ], Ql[ESDG_MAXNQ][ESDG_MAXNQ];
+  int Wh[ESDG_MAXNQ], Wl[ESDG_MAXNQ];
+  int w0h, w0l, wm;  // 2^wm >= 1/w_0
+  long long rnd[2];  // rounding constants of the products (Round)
 };
 
 struct EsdgPhys {
@@ -333,6 +342,7 @@ struct EsdgVolArgs {
   double* rhs;           // mode 0: right-hand side output
   const void* vgeo;      // [E][11][np] double (FP64) or float (mixed)
   const double* vgeo64;  // [E][11][np] double (geopotential for the pressure recovery)
+  const double* Ja;      // [E][3][3][np] (FP64 volume kernel: elements outside its fixed-point range)
   const void* fflux;     // face fluxes, double or float
   const double* x;       // coordinates (Coriolis parameter)
   const double* bg;      // mixed mode with a background: [E][3][np] rho_bg, E_bg, phi (else null)
@@ -358,6 +368,7 @@ struct EsdgMember {
   EsdgVolArgs a;       // q_in == q_io: the member's state; dq, geometry, face fluxes, dt
   const double* fgeo;  // face geometry
   const double* bg;    // mixed background (rho_bg, b_bg, p_bg, for the faces) or null
+  void* pad;
   // (sizeof a multiple of 16 bytes: the pipelined kernels bulk-copy descriptors)
 };
 

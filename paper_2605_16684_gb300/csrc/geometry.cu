@@ -8,6 +8,7 @@
 // Eq. (nm:semi)).  One CTA per element, one thread per node.
 #include "dd.cuh"
 #include "esdg_internal.cuh"
+#include "volume_fx.cuh"
 
 namespace {
 
@@ -122,6 +123,23 @@ __global__ void k_geometry(EsdgGrid g, EsdgLGL L, EsdgPhys P, double* __restrict
       }
     }
   }
+  // the FP64 path's metric terms in limbs of the element's common scale
+  __shared__ unsigned top;
+  if (threadIdx.x == 0) top = 0u;
+  __syncthreads();
+  double* vg = vgeo + (size_t)e * ESDG_NVGEO * np;
+  unsigned hi = 0u;
+  for (int k = threadIdx.x; k < 3 * np; k += blockDim.x) {
+    const double* a = vg + (size_t)(k / np) * 3 * np + k % np;
+    hi = max(hi, (unsigned)__double2hiint(a[0] * a[0] + a[np] * a[np] + a[2 * np] * a[2 * np]) & 0x7fffffffu);
+  }
+  atomicMax(&top, hi);
+  __syncthreads();
+  const int sn = esdg_fx::metric_scale(top);
+  if (threadIdx.x == 0) esdg_fx::metric_scales(vgeo, g.E, np)[e] = sn;
+  if (sn == esdg_fx::FX_NO_METRIC) return;
+  for (int k = threadIdx.x; k < 9 * np; k += blockDim.x)
+    esdg_fx::st_fx(vg + k, esdg_fx::to_fx(vg[k], sn));
 }
 
 // Face normals from the metric of the element on the face's "-" side (or the

@@ -11,6 +11,7 @@
 #include <cstring>
 
 #include "esdg_internal.cuh"
+#include "volume_fx.cuh"
 
 namespace {
 
@@ -61,10 +62,23 @@ int esdg_lgl_build(int N, EsdgLGL* out) {
       if (k != j) prod *= (x[j] - x[k]);
     lam[j] = 1.0L / prod;
   }
+  // limbs h 2^30 + l, |l| <= 2^29, of v 2^s rounded to an integer
+  auto limbs = [](long double v, int s, int* h, int* l) {
+    const long long t = std::llrint(std::ldexp(v, s));
+    const long long hh = (t + (1ll << 29)) >> 30;
+    *h = (int)hh;
+    *l = (int)(t - hh * (1ll << 30));
+  };
   out->N = N;
+  out->rnd[0] = esdg_fx::RND;
+  out->rnd[1] = esdg_fx::RNDL;
+  while ((1 << out->wm) < N * (N + 1) / 2) out->wm++;  // 1/w_0 = N (N + 1)/2
+  limbs(2.0L / ((long double)N * (N + 1)), 59 + out->wm, &out->w0h, &out->w0l);
   for (int i = 0; i < Nq; i++) {
     long double P, dP, d2P;
     legendre_all(N, x[i], &P, &dP, &d2P);
+    const long double wi = 2.0L / ((long double)N * (N + 1) * P * P);
+    limbs(1.0L / wi, 60 - out->wm, &out->Wh[i], &out->Wl[i]);
     out->xi[i] = (double)x[i];
     out->xi_lo[i] = (double)(x[i] - (long double)out->xi[i]);
     out->w[i] = (double)(2.0L / ((long double)N * (N + 1) * P * P));
@@ -75,6 +89,7 @@ int esdg_lgl_build(int N, EsdgLGL* out) {
       out->D[i][j] = (double)dij;
       out->D_lo[i][j] = (double)(dij - (long double)out->D[i][j]);
       out->Dt[i][j] = (double)(2.0L * dij);
+      limbs(2.0L * wi * dij, 59, &out->Qh[i][j], &out->Ql[i][j]);
       diag -= dij;
     }
     out->D[i][i] = (double)diag;

@@ -47,17 +47,17 @@ int batch_variant(int what, int variant, const EsdgMember* members, const int2* 
   if (variant < 0 || variant >= nk) return -1;
   switch (kinds[variant]) {
     case 0:
-      if constexpr (pipe_ok) return esdg_vol::pipe_batch<NN, true>(what, members, tiles, ntiles, grid, L, A, B, s);
+      if constexpr (pipe_ok) return esdg_vol::pipe_batch<NN>(what, members, tiles, ntiles, grid, L, A, B, s);
       return -1;
     case 1:
-      if (what == 0) return esdg_vol::launch_batch_one<NN, true, true, 0>(members, tiles, ntiles, grid, L, A, B, s) == cudaSuccess ? 0 : -1;
+      if (what == 0) return esdg_vol::launch_batch_one<NN, true, 0>(members, tiles, ntiles, grid, L, A, B, s) == cudaSuccess ? 0 : -1;
       if (what == 1) return esdg_vol::Shape<NN, true, true, 0>::EPB;
-      return esdg_vol::batch_occupancy<NN, true, true, 0>();
+      return esdg_vol::batch_occupancy<NN, true, 0>();
     default:
       if constexpr (alt_ok) {
-        if (what == 0) return esdg_vol::launch_batch_one<NN, true, true, Alt32<NN>::EPB>(members, tiles, ntiles, grid, L, A, B, s) == cudaSuccess ? 0 : -1;
+        if (what == 0) return esdg_vol::launch_batch_one<NN, true, Alt32<NN>::EPB>(members, tiles, ntiles, grid, L, A, B, s) == cudaSuccess ? 0 : -1;
         if (what == 1) return esdg_vol::Shape<NN, true, true, Alt32<NN>::EPB>::EPB;
-        return esdg_vol::batch_occupancy<NN, true, true, Alt32<NN>::EPB>();
+        return esdg_vol::batch_occupancy<NN, true, Alt32<NN>::EPB>();
       }
       return -1;
   }

@@ -9,7 +9,7 @@ cudaError_t esdg_launch_volume_mixed_moving(const EsdgGrid& g, const EsdgLGL& L,
   using namespace esdg_vol;
 #define ESDG_MV(NN)                                                                   \
   case NN:                                                                            \
-    return mode ? launch_one<NN, true, 1, 2>(g, P, L, a, s) : launch_one<NN, true, 0, 2>(g, P, L, a, s);
+    return mode ? launch_one<NN, 1, 2>(g, P, L, a, s) : launch_one<NN, 0, 2>(g, P, L, a, s);
   switch (g.N) {
     ESDG_MV(1)
     ESDG_MV(2)

@@ -1,6 +1,5 @@
 // volume64.cu -- FP64 instantiations of the flux-differencing volume kernel:
-// single-mesh launches and the batched variants (pipelined persistent kernel,
-// per-tile kernel at two tile shapes).
+// single-mesh launches and the batched kernel.
 #include "volume_impl.cuh"
 
 int esdg_volume_f64_take_timeout() {
@@ -19,45 +18,13 @@ cudaError_t esdg_launch_volume_f64(const EsdgGrid& g, const EsdgLGL& L, const Es
 }
 
 namespace {
-// alternative tile shapes (elements per CTA) offered to the batch autotuner
-template <int N> struct Alt64 { static constexpr int EPB = 0; };
-template <> struct Alt64<1> { static constexpr int EPB = 4; };
-template <> struct Alt64<2> { static constexpr int EPB = 8; };
-template <> struct Alt64<3> { static constexpr int EPB = 4; };
-template <> struct Alt64<4> { static constexpr int EPB = 3; };
-}  // namespace
-
-namespace {
-// Batched volume variants offered to the autotuner, in order: the pipelined
-// persistent kernel (when its tile fits in shared memory), the per-tile kernel
-// at the default tile shape, and at the alternative shape (when there is one).
+// The batched volume kernel has one variant.
 template <int NN>
 int batch_variant(int what, int variant, const EsdgMember* members, const int2* tiles,
                   const int* ntiles, int grid, const EsdgLGL& L, double A, double B, cudaStream_t s) {
-  constexpr bool pipe_ok = esdg_vol::Pipe64<NN, 1>::SMEM <= ESDG_PIPE_SMEM_MAX;
-  constexpr bool alt_ok = Alt64<NN>::EPB > 0;
-  int kinds[3], nk = 0;
-  if (pipe_ok) kinds[nk++] = 0;
-  kinds[nk++] = 1;
-  if (alt_ok) kinds[nk++] = 2;
-  if (what == 3) return nk;
-  if (variant < 0 || variant >= nk) return -1;
-  switch (kinds[variant]) {
-    case 0:
-      if constexpr (pipe_ok) return esdg_vol::pipe_batch<NN, false>(what, members, tiles, ntiles, grid, L, A, B, s);
-      return -1;
-    case 1:
-      if (what == 0) return esdg_vol::launch_batch_one<NN, false, false, 0>(members, tiles, ntiles, grid, L, A, B, s) == cudaSuccess ? 0 : -1;
-      if (what == 1) return esdg_vol::Shape<NN, false, false, 0>::EPB;
-      return esdg_vol::batch_occupancy<NN, false, false, 0>();
-    default:
-      if constexpr (alt_ok) {
-        if (what == 0) return esdg_vol::launch_batch_one<NN, false, false, Alt64<NN>::EPB>(members, tiles, ntiles, grid, L, A, B, s) == cudaSuccess ? 0 : -1;
-        if (what == 1) return esdg_vol::Shape<NN, false, false, Alt64<NN>::EPB>::EPB;
-        return esdg_vol::batch_occupancy<NN, false, false, Alt64<NN>::EPB>();
-      }
-      return -1;
-  }
+  if (what == 3) return 1;
+  if (variant != 0) return -1;
+  return esdg_vol::batch_volume64<NN>(what, members, tiles, ntiles, grid, L, A, B, s);
 }
 
 int batch_dispatch(int what, int N, int variant, const EsdgMember* members, const int2* tiles,

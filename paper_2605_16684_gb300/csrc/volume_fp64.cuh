@@ -1,0 +1,389 @@
+// volume_fp64.cuh -- the FP64 volume kernel: persistent CTAs of a few elements,
+// pairs in fixed point (volume_fx.cuh) or, for elements outside its range, FP64.
+//
+// A tile's phases use different pipes: the prologue and the epilogue the FP64
+// pipe and memory, the pair pass the integer pipes.  The tile is therefore
+// small (about 192 threads) and several CTAs share an SM, so that one CTA's
+// prologue and epilogue run under another's pair pass.
+#pragma once
+#include "volume_pipe.cuh"
+
+namespace esdg_vol {
+
+// Elements per tile and the CTAs planned per SM (MINB; it sets the register
+// budget).  Measured at N = 4, 32^3: two elements and three CTAs (128 registers)
+// 1.21 ms, two CTAs (168 registers) 1.29 ms, one element and five CTAs (a third of
+// the third warp idle) 1.49 ms, four elements and one CTA 1.50 ms.  N = 5: two
+// elements (216 of 224 lanes) 0.513 ms against one (108 of 128) 0.526 ms at 20^3.
+template <int N> struct F64Cfg;
+template <> struct F64Cfg<1> { static constexpr int EPB = 16, MINB = 2; };
+template <> struct F64Cfg<2> { static constexpr int EPB = 7, MINB = 2; };
+template <> struct F64Cfg<3> { static constexpr int EPB = 4, MINB = 2; };
+template <> struct F64Cfg<4> { static constexpr int EPB = 2, MINB = 3; };
+template <> struct F64Cfg<5> { static constexpr int EPB = 2, MINB = 2; };
+template <> struct F64Cfg<6> { static constexpr int EPB = 1, MINB = 2; };
+template <> struct F64Cfg<7> { static constexpr int EPB = 1, MINB = 2; };
+
+template <int N>
+struct F64 {
+  using SH = Shape<N, false, 0, F64Cfg<N>::EPB>;
+  static constexpr int P = SH::NP * SH::EPB;  // nodes per tile
+  static constexpr int NF = SH::NF + 1;
+  static constexpr int S0 = 0;                // [el][NF][NP] node fields; sums (1..3) in the Ja slots
+  // [el][6][NP] sums 0 and 4; first the copy of q (a bulk-copy target: 16-byte aligned)
+  static constexpr int X0 = (NF * P + 1) / 2 * 2;
+  static constexpr size_t SMEM = sizeof(double) * (size_t)(X0 + 6 * P + 4);
+  static_assert(SH::NF == 18, "FP64 node fields");
+};
+
+struct OneIssuer {  // thread 0 issues the copies
+  static constexpr int FIRST = 0, COUNT = 1;
+  static __device__ __forceinline__ unsigned mask() { return 1u; }
+};
+
+// All pairs of one pencil.  Node i is paired with the nodes after it; its sum
+// is then complete, leaves through done(i, sum) and the sums move down by one,
+// so that the code holds N pair bodies instead of N (N + 1)/2.
+template <int N, typename R, typename LOAD, typename PAIR, typename DONE>
+__device__ __forceinline__ void pencil_rolled(R (&acc)[N + 1][5], const LOAD& load,
+                                              const PAIR& pair, const DONE& done) {
+  constexpr int Nq = N + 1;
+#pragma unroll 1
+  for (int i = 0; i < Nq; i++) {
+    const auto A = load(i);
+#pragma unroll
+    for (int k = 1; k < Nq; k++) {
+      if (i + k < Nq) {
+        const auto B = load(i + k);
+        pair(A, B, i, i + k, acc[0], acc[k]);
+      }
+    }
+    done(i, acc[0]);
+#pragma unroll
+    for (int k = 0; k < N; k++)
+#pragma unroll
+      for (int v = 0; v < 5; v++) acc[k][v] = acc[k + 1][v];
+  }
+}
+
+template <int N, int MODE, bool TABLE>
+__global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
+    k_volume64(const EsdgMember one, const EsdgMember* __restrict__ members,
+               const int2* __restrict__ tiles, const int* __restrict__ ntiles_d, int ntiles_1,
+               const __grid_constant__ EsdgLGL L, double rkA, double rkB, unsigned phantom, int t1,
+               int s1) {
+  static_assert(!TABLE || MODE == 1, "the batched kernel applies an RK stage");
+  using SH = typename F64<N>::SH;
+  constexpr int Nq = SH::Nq, NP = SH::NP, NPEN = SH::NPEN, EPB = SH::EPB, NF = F64<N>::NF;
+  constexpr int T = SH::THREADS;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ __align__(16) EsdgMember M;
+  __shared__ unsigned long long bar;
+  __shared__ esdg_fx::FxElement fxe[EPB];
+  // per element: its path; the pencils (three directions, 64
+  // bits) whose interface terms leave its range
+  __shared__ unsigned gen[EPB], far_lift[EPB][3][2];
+  double* const sm = reinterpret_cast<double*>(smraw) + F64<N>::S0;
+  double* const xs = reinterpret_cast<double*>(smraw) + F64<N>::X0;
+  const int tid = threadIdx.x;
+  const int ntiles = TABLE ? *ntiles_d : ntiles_1;
+  int member = -1;
+  if (tid == 0) {
+    esdg_mbar_init(&bar, 1);
+    esdg_fence_mbar_init();
+    if constexpr (!TABLE) M = one;
+  }
+  __syncthreads();
+  unsigned parity = 0;
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, parity ^= 1u) {
+    if constexpr (TABLE) {
+      const int m = tiles[tile].x;
+      if (m != member) {
+        const int* src = reinterpret_cast<const int*>(members + m);
+        int* dst = reinterpret_cast<int*>(&M);
+        for (int k = tid; k < (int)(sizeof(EsdgMember) / sizeof(int)); k += T) dst[k] = src[k];
+        member = m;
+        __syncthreads();
+      }
+    }
+    const EsdgGrid& g = M.g;
+    const EsdgPhys& P = M.P;
+    const EsdgVolArgs& a = M.a;
+    const int4 tr = pipe_tile<TABLE, EPB>(tiles, tile, t1, s1, g.E);
+    const int e0 = tr.y, ne = tr.z;
+    const double* const vg = reinterpret_cast<const double*>(a.vgeo);
+    const int* const nscale = esdg_fx::metric_scales(vg, g.E, NP);
+    if (tid == 0) {
+      const double* q = a.q_in + (size_t)e0 * 5 * NP;
+      const BlockCopy bl[1] = {{xs, q, a.q_in + (size_t)g.E * 5 * NP, ne * 5 * NP, 8}};
+      pipe_issue<OneIssuer>(0, bl, 1, &bar, 0, nullptr, nullptr, phantom);
+      phantom = 0;
+    }
+    if (tid < EPB) {
+      fxe[tid].mu = fxe[tid].mf = 0u;
+      gen[tid] = 0u;
+      for (int w = 0; w < 6; w++) far_lift[tid][w / 2][w % 2] = 0u;
+    }
+    // the metric limbs and (in the spare field) the geopotential
+    for (int idx = tid; idx < ne * NP; idx += T) {
+      const int el = idx / NP, n = idx - el * NP;
+      double* S = sm + (size_t)el * NF * NP + n;
+      const double* gr = vg + (size_t)(e0 + el) * ESDG_NVGEO * NP + n;
+#pragma unroll
+      for (int k = 0; k < 9; k++) esdg_cp_async(S + (SH::F_NH + k) * NP, gr + k * NP);
+      esdg_cp_async(S + 18 * NP, gr + 10 * NP);
+    }
+    esdg_cp_async_wait_all();  // these, and thread 0's edge elements of q
+    const bool ok = esdg_mbar_wait(&bar, parity, ESDG_WAIT_LIMIT);
+    if (__syncthreads_or(!ok)) {
+      if (tid == 0) atomicExch(&g_esdg_vol_timeout, 1);
+      return;
+    }
+    // ---- prologue: node fields (FP64) and the elements' largest values ------------
+    {
+      const double* qr0 = xs + esdg_block_shift(a.q_in + (size_t)e0 * 5 * NP);
+      const double gm1 = P.gamma - 1.0;
+      auto mag = [](double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; };
+      for (int idx = tid; idx < ne * NP; idx += T) {
+        const int el = idx / NP, n = idx - el * NP;
+        double* S = sm + (size_t)el * NF * NP;
+        const double* qr = qr0 + (size_t)el * 5 * NP;
+        prims64<NP>(qr[n], qr[NP + n], qr[2 * NP + n], qr[3 * NP + n], qr[4 * NP + n],
+                    S[18 * NP + n], gm1, S, n);
+        atomicMax(&fxe[el].mu, max(mag(S[3 * NP + n]), max(mag(S[4 * NP + n]), mag(S[5 * NP + n]))));
+        atomicMax(&fxe[el].mf, mag(S[6 * NP + n]));
+      }
+    }
+    __syncthreads();  // the copy of q consumed
+    // ---- which elements take the fixed-point pairs, and their scales ---------------
+    for (int idx = tid; idx < ne * NP; idx += T) {
+      const int el = idx / NP, n = idx - el * NP;
+      const double* S = sm + (size_t)el * NF * NP;
+      const unsigned path = esdg_fx::fx_path(S[n], S[2 * NP + n], S[0], S[2 * NP]);
+      if (path != esdg_fx::FX_NARROW) atomicMax(&gen[el], path);
+      if (n == 0) {
+        esdg_fx::fx_scales(fxe[el], S[0], S[2 * NP], nscale[e0 + el], P.gamma - 1.0, P.igm1, L.wm);
+        if (!fxe[el].sc.ok) atomicMax(&gen[el], (unsigned)esdg_fx::FX_GENERAL);
+      }
+    }
+    __syncthreads();
+    for (int idx = tid; idx < ne * NP; idx += T) {
+      const int el = idx / NP, n = idx - el * NP;
+      double* S = sm + (size_t)el * NF * NP;
+      if (gen[el] == esdg_fx::FX_GENERAL) prims64_general<NP>(S, n, a.Ja + (size_t)(e0 + el) * 9 * NP);
+      else esdg_fx::fx_convert<NP>(S, n, fxe[el], gen[el], 0.5 * P.igm1);
+    }
+    __syncthreads();
+
+    // ---- pair pass: this thread's pencil --------------------------------------------
+    bool far = false;
+    const int el = tid / (3 * NPEN);
+    if (tid < SH::PENCILS && el < ne) {
+      const int rr = tid - el * 3 * NPEN;
+      const int d = rr / NPEN;
+      const int pen = rr - d * NPEN;
+      const int ps = pen % Nq, pt = pen / Nq;
+      const int stride = (d == 0) ? 1 : ((d == 1) ? Nq : Nq * Nq);
+      const int base = (d == 0) ? Nq * (ps + Nq * pt) : ((d == 1) ? (ps + Nq * Nq * pt) : (ps + Nq * pt));
+      double* const S = sm + (size_t)el * NF * NP;
+      // this pencil's sums leave through its own Ja slots (momentum) and the
+      // spare slots (mass, energy) as the nodes complete
+      double* const om = S + (SH::F_NH + 3 * d) * NP + base;
+      double* const ox = xs + ((size_t)el * 6 + 2 * d) * NP + base;
+      const FaceTerms<double> ft = face_fetch<N, double>(g, a, e0 + el, d, ps + Nq * pt);
+      if (gen[el] != esdg_fx::FX_GENERAL) {
+        using esdg_fx::i64;
+        const esdg_fx::FxElement& E2 = fxe[el];
+        const int ks = E2.sc.s1;
+        i64 acc[Nq][5];
+#pragma unroll
+        for (int v = 0; v < 5; v++) {
+          const int so = E2.out[v == 0 ? 0 : (v == 4 ? 2 : 1)];
+          far |= esdg_fx::fx_over(ft.m[v], so, 3) || esdg_fx::fx_over(ft.p[v], so, 3);
+#pragma unroll
+          for (int i = 0; i < Nq; i++) acc[i][v] = 0;
+          acc[0][v] = -esdg_fx::fx_lift(ft.m[v], so, L);
+          acc[N][v] = esdg_fx::fx_lift(ft.p[v], so, L);
+        }
+        if (far) {  // the epilogue adds them in FP64
+          atomicOr(&far_lift[el][d][pen >> 5], 1u << (pen & 31));
+#pragma unroll
+          for (int v = 0; v < 5; v++) acc[0][v] = acc[N][v] = 0;
+        }
+        const auto load = [&](int i) { return esdg_fx::fx_load<NP>(S, base + i * stride, d); };
+        const auto done = [&](int i, const i64* s) {
+          auto out = [&](int v) {
+            return __longlong_as_double(
+                esdg_fx::mul(esdg_fx::limbs4(s[v]), esdg_fx::Fx{L.Wh[i], L.Wl[i]}, L.rnd[0]));
+          };
+          const int n = i * stride;
+          ox[n] = out(0);
+          ox[NP + n] = out(4);
+          om[n] = out(1);
+          om[NP + n] = out(2);
+          om[2 * NP + n] = out(3);
+        };
+        auto pass = [&](auto path) {
+          pencil_rolled<N>(acc, load,
+                           [&](const esdg_fx::FxNode& A, const esdg_fx::FxNode& B, int i, int l,
+                               i64* ai, i64* al) {
+                             esdg_fx::pair_fx<decltype(path)::value>(
+                                 A, B, esdg_fx::Fx{L.Qh[i][l], L.Ql[i][l]}, ks,
+                                 esdg_fx::Round{L.rnd[0], L.rnd[1]}, ai, al);
+                           }, done);
+        };
+        using namespace esdg_fx;
+        if (gen[el] == FX_NARROW) pass(std::integral_constant<int, FX_NARROW>{});
+        else if (gen[el] == FX_WIDE) pass(std::integral_constant<int, FX_WIDE>{});
+        else pass(std::integral_constant<int, FX_TALL>{});
+      } else {
+        double acc[Nq][5];
+#pragma unroll
+        for (int i = 0; i < Nq; i++)
+#pragma unroll
+          for (int v = 0; v < 5; v++) acc[i][v] = i == 0 ? -ft.m[v] : (i == N ? ft.p[v] : 0.0);
+        const CeSeries cs = ce_series(0.5 * P.igm1);
+        pencil_rolled<N>(
+            acc,
+            [&](int i) { return load_node<double, true, SH::F_NH, NP, 0>(S, base + i * stride, d); },
+            [&](const Node<double>& A, const Node<double>& B, int i, int l, double* ai, double* al) {
+              pair64<true>(A, B, L.Dt[i][l], L.Dt[l][i], cs, ai, al);
+            },
+            [&](int i, const double* s) {
+              const int n = i * stride;
+              ox[n] = s[0];
+              ox[NP + n] = s[4];
+              om[n] = s[1];
+              om[NP + n] = s[2];
+              om[2 * NP + n] = s[3];
+            });
+      }
+    }
+    const bool any_far = __syncthreads_or(far);
+
+    // ---- epilogue ------------------------------------------------------------------
+    const double dt = a.dt;
+    const double* const qin = a.q_in;
+    double* const dqp = reinterpret_cast<double*>(a.dq);
+    double* const qio = a.q_io;
+    double* const rhsp = a.rhs;
+    bool bad = false;
+    const bool rot = P.f0 != 0.0 || P.beta != 0.0;
+    // one thread per node; the loads of two nodes are in flight together
+    struct Old {
+      double q[5], d[5], iJ, y;
+    };
+    auto fetch = [&](int idx) {
+      const int el2 = idx / NP, n = idx - el2 * NP, e2 = e0 + el2;
+      const size_t qv = (size_t)e2 * 5 * NP + n;
+      Old o;
+      o.iJ = vg[((size_t)e2 * ESDG_NVGEO + 9) * NP + n];
+#pragma unroll
+      for (int v = 0; v < 5; v++) {
+        if (MODE != 0 || (rot && (v == 1 || v == 2))) o.q[v] = qin[qv + v * NP];
+        if (MODE != 0 && rkA != 0.0) o.d[v] = dqp[qv + v * NP];
+      }
+      if (rot) o.y = a.x[((size_t)e2 * 3 + 1) * NP + n];
+      return o;
+    };
+    auto update = [&](int idx, const Old& o) {
+      const int el2 = idx / NP, n = idx - el2 * NP, e2 = e0 + el2;
+      const size_t qv = (size_t)e2 * 5 * NP + n;
+      const bool general = gen[el2] == esdg_fx::FX_GENERAL;
+      // -1/J, times dt for a stage update (r then holds dt times the right-hand side)
+      const double sJ = MODE != 0 ? -o.iJ * dt : -o.iJ;
+      double f = 0.0;
+      if (rot) {
+        f = P.f0 + P.beta * (o.y - P.y0);
+        if (MODE != 0) f *= dt;
+      }
+#pragma unroll
+      for (int v = 0; v < 5; v++) {
+        const bool mom = v >= 1 && v <= 3;
+        const double* Z = mom ? sm + ((size_t)el2 * NF + SH::F_NH + v - 1) * NP + n
+                              : xs + ((size_t)el2 * 6 + (v ? 1 : 0)) * NP + n;
+        const int zs = mom ? 3 * NP : 2 * NP;
+        const double z0 = Z[0], z1 = Z[zs], z2 = Z[2 * zs];
+        double r;
+        if (!general) {
+          // the power of two on the exponent of the scale factor
+          const int so = fxe[el2].out[v == 0 ? 0 : (v == 4 ? 2 : 1)];
+          const double ss = __hiloint2double(__double2hiint(sJ) - so * (1 << 20), __double2loint(sJ));
+          r = ss * (double)(__double_as_longlong(z0) + __double_as_longlong(z1) +
+                            __double_as_longlong(z2));
+          if (any_far) r = fma(sJ, far_terms<N>(g, a, e2, n, v, far_lift[el2]), r);
+        } else {
+          r = sJ * (z0 + z1 + z2);
+        }
+        if (rot && v == 1) r = fma(f, o.q[2], r);
+        if (rot && v == 2) r = fma(-f, o.q[1], r);
+        if constexpr (MODE == 0) {
+          rhsp[qv + v * NP] = r;
+        } else {
+          // first stage (A = 0): the register is not read (see stage32)
+          const double dv = rkA == 0.0 ? r : fma(rkA, o.d[v], r);
+          dqp[qv + v * NP] = dv;
+          const double qn = fma(rkB, dv, o.q[v]);
+          qio[qv + v * NP] = qn;
+          bad |= esdg_bad_state(qn, v == 0);
+        }
+      }
+    };
+    for (int i0 = tid; i0 < ne * NP; i0 += 2 * T) {
+      const int i1 = i0 + T;
+      const Old o0 = fetch(i0), o1 = fetch(i1 < ne * NP ? i1 : i0);
+      update(i0, o0);
+      if (i1 < ne * NP) update(i1, o1);
+    }
+    if (MODE != 0 && bad && a.status) *a.status = 1;
+    __syncthreads();  // the sums and the element data read
+  }
+}
+
+template <int N, int MODE>
+cudaError_t launch_volume64(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL& L,
+                            const EsdgVolArgs& a, cudaStream_t s) {
+  using SH = typename F64<N>::SH;
+  constexpr auto k = k_volume64<N, MODE, false>;
+  const int cap = pipe_grid_cap<k>(SH::THREADS, F64<N>::SMEM);
+  if (cap < 0) return cudaErrorInvalidConfiguration;
+  int ntiles, grid, t1, s1;
+  pipe_split(g.E, SH::EPB, cap, ntiles, grid, t1, s1);
+  if (ntiles == 0) return cudaSuccess;
+  k<<<grid, SH::THREADS, F64<N>::SMEM, s>>>(pipe_member(g, P, a), nullptr, nullptr, nullptr, ntiles,
+                                            L, a.rkA, a.rkB, esdg_take_phantom(), t1, s1);
+  return cudaGetLastError();
+}
+
+// batched (TABLE) launches; what: 0 launch (0 / -1), 1 elements per tile, 2 CTAs per SM
+template <int N>
+int batch_volume64(int what, const EsdgMember* members, const int2* tiles, const int* ntiles,
+                   int grid, const EsdgLGL& L, double A, double B, cudaStream_t s) {
+  using SH = typename F64<N>::SH;
+  constexpr auto k = k_volume64<N, 1, true>;
+  if (what == 1) return SH::EPB;
+  if (what == 2) {
+    int nb = 0;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F64<N>::SMEM) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, SH::THREADS, F64<N>::SMEM) !=
+            cudaSuccess) {
+      cudaGetLastError();
+      return 1;
+    }
+    return nb > 0 ? nb : 1;
+  }
+  static bool configured = false;  // one-time attribute set per instantiation
+  if (!configured) {
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F64<N>::SMEM) !=
+        cudaSuccess)
+      return -1;
+    configured = true;
+  }
+  EsdgMember none;
+  memset(&none, 0, sizeof(none));
+  k<<<grid, SH::THREADS, F64<N>::SMEM, s>>>(none, members, tiles, ntiles, 0, L, A, B, 0u, 0, 0);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+}  // namespace esdg_vol

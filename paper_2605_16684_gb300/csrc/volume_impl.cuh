@@ -33,6 +33,7 @@
 // sums and face lifts run in FP32; the log branch uses log1pf of the ratio;
 // the geopotential is carried relative to each element's first node.
 #pragma once
+#include "volume_fp64.cuh"
 #include "volume_pipe.cuh"
 #include "volume_tile.cuh"
 #include "volume_ws.cuh"
@@ -45,8 +46,8 @@ cudaError_t launch_volume_t(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys&
 #define ESDG_CASE(NN)                                                          \
   case NN:                                                                     \
     if constexpr (!MIXED) {                                                    \
-      return mode ? launch_pipe64<NN, 1>(g, P, L, a, s)                        \
-                  : launch_pipe64<NN, 0>(g, P, L, a, s);                       \
+      return mode ? launch_volume64<NN, 1>(g, P, L, a, s)                        \
+                  : launch_volume64<NN, 0>(g, P, L, a, s);                       \
     }                                                                          \
     if constexpr (MIXED) {                                                     \
       if (a.bg && a.bgq) return esdg_launch_volume_mixed_moving(g, L, P, mode, a, s); \
@@ -57,11 +58,11 @@ cudaError_t launch_volume_t(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys&
         if constexpr (Pipe32<NN, 1>::SMEM <= ESDG_PIPE_SMEM_MAX)               \
           return mode ? launch_pipe32<NN, 1>(g, P, L, a, s)                    \
                       : launch_pipe32<NN, 0>(g, P, L, a, s);                   \
-        return mode ? launch_one<NN, MIXED, 1, true>(g, P, L, a, s)            \
-                    : launch_one<NN, MIXED, 0, true>(g, P, L, a, s);           \
+        return mode ? launch_one<NN, 1, true>(g, P, L, a, s)            \
+                    : launch_one<NN, 0, true>(g, P, L, a, s);           \
       }                                                                        \
-      return mode ? launch_one<NN, MIXED, 1, false>(g, P, L, a, s)             \
-                  : launch_one<NN, MIXED, 0, false>(g, P, L, a, s);            \
+      return mode ? launch_one<NN, 1, false>(g, P, L, a, s)             \
+                  : launch_one<NN, 0, false>(g, P, L, a, s);            \
     }
   switch (g.N) {
     ESDG_CASE(1)

@@ -9,34 +9,28 @@
 #include <type_traits>
 
 #include "esdg_internal.cuh"
+#include "volume_fx.cuh"
 
 namespace esdg_vol {
 
 
-template <int N, bool MIXED>
-struct Cfg;
-// elements per CTA, chosen so that 3 Nq^2 EPB pencils fill whole warps
-template <> struct Cfg<1, false> { static constexpr int EPB = 8; };
-template <> struct Cfg<2, false> { static constexpr int EPB = 16; };
-template <> struct Cfg<3, false> { static constexpr int EPB = 8; };
-template <> struct Cfg<4, false> { static constexpr int EPB = 5; };
-template <> struct Cfg<5, false> { static constexpr int EPB = 2; };
-template <> struct Cfg<6, false> { static constexpr int EPB = 1; };
-template <> struct Cfg<7, false> { static constexpr int EPB = 1; };
-template <> struct Cfg<1, true> { static constexpr int EPB = 16; };
-template <> struct Cfg<2, true> { static constexpr int EPB = 16; };
-template <> struct Cfg<3, true> { static constexpr int EPB = 8; };
-template <> struct Cfg<4, true> { static constexpr int EPB = 5; };
-template <> struct Cfg<5, true> { static constexpr int EPB = 3; };
-template <> struct Cfg<6, true> { static constexpr int EPB = 2; };
-template <> struct Cfg<7, true> { static constexpr int EPB = 2; };
+// elements per CTA of the mixed kernels, chosen so that 3 Nq^2 EPB pencils fill
+// whole warps
+template <int N> struct Cfg;
+template <> struct Cfg<1> { static constexpr int EPB = 16; };
+template <> struct Cfg<2> { static constexpr int EPB = 16; };
+template <> struct Cfg<3> { static constexpr int EPB = 8; };
+template <> struct Cfg<4> { static constexpr int EPB = 5; };
+template <> struct Cfg<5> { static constexpr int EPB = 3; };
+template <> struct Cfg<6> { static constexpr int EPB = 2; };
+template <> struct Cfg<7> { static constexpr int EPB = 2; };
 
 // BG: 0 no background, 1 a background at rest (hydrostatic), 2 a moving
 // background (one that carries a flow; mixed mode only)
 template <int N, bool MIXED, int BG = 0, int EPB_ = 0>
 struct Shape {
   static constexpr int Nq = N + 1, NP = Nq * Nq * Nq, NPEN = Nq * Nq;
-  static constexpr int EPB = EPB_ > 0 ? EPB_ : Cfg<N, MIXED>::EPB;  // elements per CTA (tile)
+  static constexpr int EPB = EPB_ > 0 ? EPB_ : Cfg<N>::EPB;  // elements per CTA (tile)
   static constexpr int PENCILS = 3 * NPEN * EPB;
   static constexpr int THREADS = ((PENCILS + 31) / 32) * 32;
   // node fields: rq=rho/4, bh=b/2, ib=1/b, uh=u/2 (3), ph=phi/2, [lr, lb], nh=Ja/2 (9),
@@ -449,29 +443,24 @@ __device__ __forceinline__ void pair32bgm(const Node<float>& A, const Node<float
   al[4] = fmaf(dli, FE, al[4]);
 }
 
-// ce: 1/(2(gamma - 1)) as float (mixed) or as the scaled series (FP64)
-template <int N, bool MIXED, bool LOGS, int BG, typename CE>
-__device__ __forceinline__ void pencil_pass(const typename Shape<N, MIXED, BG>::R* __restrict__ S,
-                                            int d, int base, int stride, const EsdgLGL& L,
-                                            const CE& ce,
-                                            typename Shape<N, MIXED, BG>::R (&acc)[N + 1][5]) {
-  using SH = Shape<N, MIXED, BG>;
-  using R = typename SH::R;
+// every pair of one pencil in FP32; ce = 1/(2(gamma - 1))
+template <int N, bool LOGS, int BG>
+__device__ __forceinline__ void pencil_pass(const float* __restrict__ S, int d, int base, int stride,
+                                            const EsdgLGL& L, float ce, float (&acc)[N + 1][5]) {
+  using SH = Shape<N, true, BG>;
   constexpr int Nq = N + 1;
 #pragma unroll
   for (int i = 0; i < Nq; i++) {
-    const Node<R> A = load_node<R, LOGS, SH::F_NH, SH::NP, BG>(S, base + i * stride, d);
+    const Node<float> A = load_node<float, LOGS, SH::F_NH, SH::NP, BG>(S, base + i * stride, d);
 #pragma unroll
     for (int l = i + 1; l < Nq; l++) {
-      const Node<R> B = load_node<R, LOGS, SH::F_NH, SH::NP, BG>(S, base + l * stride, d);
-      if constexpr (MIXED && BG == 2)
+      const Node<float> B = load_node<float, LOGS, SH::F_NH, SH::NP, BG>(S, base + l * stride, d);
+      if constexpr (BG == 2)
         pair32bgm<LOGS>(A, B, L.Dtf[i][l], L.Dtf[l][i], ce, acc[i], acc[l]);
-      else if constexpr (MIXED && BG)
+      else if constexpr (BG)
         pair32bg<LOGS>(A, B, L.Dtf[i][l], L.Dtf[l][i], ce, acc[i], acc[l]);
-      else if constexpr (MIXED)
-        pair32<LOGS>(A, B, L.Dtf[i][l], L.Dtf[l][i], ce, acc[i], acc[l]);
       else
-        pair64<LOGS>(A, B, L.Dt[i][l], L.Dt[l][i], ce, acc[i], acc[l]);
+        pair32<LOGS>(A, B, L.Dtf[i][l], L.Dtf[l][i], ce, acc[i], acc[l]);
     }
   }
 }
@@ -507,6 +496,23 @@ __device__ __forceinline__ FaceTerms<R> face_fetch(const EsdgGrid& g, const Esdg
   }
   return t;
 }
+// The interface terms of one node and variable from its element's pencils in
+// the mask far (per direction, one bit per pencil), read from global memory.
+template <int N>
+__device__ double far_terms(const EsdgGrid& g, const EsdgVolArgs& a, int e, int n, int v,
+                            const unsigned (*far)[2]) {
+  constexpr int Nq = N + 1, NPEN = Nq * Nq;
+  const int c[3] = {n % Nq, (n / Nq) % Nq, n / NPEN};
+  double sum = 0.0;
+  for (int d = 0; d < 3; d++) {
+    const int fn = (d == 0 ? c[1] : c[0]) + Nq * (d == 2 ? c[1] : c[2]);
+    if ((c[d] != 0 && c[d] != N) || !((far[d][fn >> 5] >> (fn & 31)) & 1u)) continue;
+    const FaceTerms<double> t = face_fetch<N, double>(g, a, e, d, fn);
+    if (c[d] == 0) sum -= t.m[v];
+    else sum += t.p[v];
+  }
+  return sum;
+}
 // Mixed path: the terms are added after the pair sums (once the element's
 // reference geopotential is restored in them); fetched before the pair pass,
 // their gathers' latency hides behind it.
@@ -518,56 +524,38 @@ __device__ __forceinline__ void face_add(const FaceTerms<R>& t, R (&acc)[N + 1][
     acc[N][v] += t.p[v];
   }
 }
-// INIT: the terms are the accumulators' initial value (FP64: they are then
-// loaded long before their first use), else they are added at once.
-template <bool INIT, int N, typename R>
-__device__ __forceinline__ void face_lift(const EsdgGrid& g, const EsdgVolArgs& a, int e, int d,
-                                          int fn, R (&acc)[N + 1][5]) {
-  const FaceTerms<R> t = face_fetch<N, R>(g, a, e, d, fn);
-  if (INIT) {
-#pragma unroll
-    for (int v = 0; v < 5; v++) {
-      acc[0][v] = -t.m[v];
-      acc[N][v] = t.p[v];
-    }
-  } else {
-    face_add<N, R>(t, acc);
-  }
-}
-
-// FP64 node primitives from the conserved state: rho/4, b/2 = rho/(4p),
-// 1/b = 2p/rho, u/2 and phi/2, with p = (gamma - 1)(E - rho phi - |rho u|^2/(2 rho)).
-// Power-of-two factors are applied exactly on the exponent field and b/2 is
-// taken as 1/(2 (1/b)): 15 FP64-pipe instructions per node.
+// FP64 node primitives from the conserved state: rho/4, 1/b = 2p/rho, u/2,
+// phi/2 and p/2 (in the slot of ln b), with p = (gamma - 1)(E - rho phi -
+// |rho u|^2/(2 rho)).  b/2 and the logarithms follow in prims64_general for the elements that need them.
 template <int NP>
 __device__ __forceinline__ void prims64(double q0, double q1, double q2, double q3, double q4,
                                         double phi, double gm1, double* S, int n) {
   const double ir = esdg_rcp(q0);
-  const double hi = esdg_ldexp(ir, -1);  // 1/(2 rho)
+  const double hi = esdg_ldexp(ir, -1);
   const double u0 = q1 * hi, u1 = q2 * hi, u2 = q3 * hi;
   double ei = fma(-q0, phi, q4);
   ei = fma(-q1, u0, ei);
   ei = fma(-q2, u1, ei);
   ei = fma(-q3, u2, ei);
-  const double p = gm1 * ei;
-  const double ib = esdg_ldexp(p, 1) * ir;  // 1/b = 2p/rho
+  const double ph = (0.5 * gm1) * ei;  // p/2
   S[0 * NP + n] = esdg_ldexp(q0, -2);
-  S[1 * NP + n] = esdg_ldexp(esdg_rcp(ib), -1);
-  S[2 * NP + n] = ib;
+  S[2 * NP + n] = esdg_ldexp(ph, 2) * ir;  // 1/b = 2p/rho
   S[3 * NP + n] = u0;
   S[4 * NP + n] = u1;
   S[5 * NP + n] = u2;
-  S[6 * NP + n] = esdg_ldexp(phi, -1);
+  S[6 * NP + n] = 0.5 * phi;
+  S[8 * NP + n] = ph;
 }
-
-// Does any pair of this element leave the FP64 series range?  All
-// |x_n/x_0 - 1| below 0.0095 (x = rho, b) bound |f| < 0.0096 for every pair,
-// i.e. u < 1e-4.  Integer-repacked FP32 comparisons keep the FP64 pipe free.
+// the remaining fields of pair64: b/2 = 1/(2 (1/b)), ln rho, ln b, and Ja/2
+// (Ja: the element's [3][3][NP] block)
 template <int NP>
-__device__ __forceinline__ bool out_of_series64(const double* S, int n) {
-  const float r0 = esdg_d2f(S[0]), rn = esdg_d2f(S[n]);
-  const float b0 = esdg_d2f(S[NP]), bn = esdg_d2f(S[NP + n]);
-  return fabsf(rn - r0) > 0.0095f * r0 || fabsf(bn - b0) > 0.0095f * b0;
+__device__ __forceinline__ void prims64_general(double* S, int n, const double* Ja) {
+#pragma unroll
+  for (int k = 0; k < 9; k++) S[(9 + k) * NP + n] = esdg_ldexp(Ja[k * NP + n], -1);
+  const double bh = esdg_ldexp(esdg_rcp(S[2 * NP + n]), -1);
+  S[1 * NP + n] = bh;
+  S[7 * NP + n] = log(4.0 * S[n]);
+  S[8 * NP + n] = log(2.0 * bh);
 }
 
 // Mixed-precision node prologue without a background: FP32 primitives, the

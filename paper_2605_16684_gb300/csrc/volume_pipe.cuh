@@ -1,6 +1,7 @@
-// volume_pipe.cuh -- the pipelined persistent volume kernels (FP64 and mixed):
-// one CTA per SM walks its tiles while the copy engine prefetches the next
-// tile; single meshes or batch work tables; their launchers.
+// volume_pipe.cuh -- tiles, bulk copies and launch helpers of the persistent volume
+// kernels, and the pipelined mixed-precision one: one CTA per SM walks its
+// tiles while the copy engine prefetches the next tile; single meshes or batch
+// work tables.
 #pragma once
 #include "volume_pairs.cuh"
 
@@ -35,41 +36,11 @@ __device__ __forceinline__ void pipe_drain(unsigned long long* bar, unsigned par
   if (issued) esdg_mbar_wait(bar, parity, ESDG_WAIT_LIMIT);
 }
 // dynamic shared memory a pipelined tile may use (227 KB less static use)
-#define ESDG_PIPE_SMEM_MAX (232448 - 1024)
+#define ESDG_PIPE_SMEM_MAX (232448 - 4096)
 
-// Tile shape of the pipelined kernels: elements per tile (EPB) and the CTAs
-// the launch bounds plan per SM (MINB).  With MINB = 2 two CTAs share an SM,
-// so one CTA's FP64 prologue and epilogue run under the other's pair pass; at
-// N = 4 two CTAs of 2-element tiles time the same as one CTA of 5-element
-// tiles (fewer warps, more idle lanes), and 3-element tiles (8 warps, no
-// register spills) are 8 % slower, so the default stays EPB = 5, MINB = 1.
-#ifndef ESDG_PIPE4_EPB64
-#define ESDG_PIPE4_EPB64 5
-#endif
-#ifndef ESDG_PIPE4_MINB64
-#define ESDG_PIPE4_MINB64 1
-#endif
-#ifndef ESDG_PIPE4_EPB32
-#define ESDG_PIPE4_EPB32 5
-#endif
-#ifndef ESDG_PIPE4_MINB32
-#define ESDG_PIPE4_MINB32 1
-#endif
-template <int N, bool MIXED>
-struct PipeCfg {
-  static constexpr int EPB = Cfg<N, MIXED>::EPB, MINB = 1;
-};
-template <>
-struct PipeCfg<4, false> {
-  static constexpr int EPB = ESDG_PIPE4_EPB64, MINB = ESDG_PIPE4_MINB64;
-};
-template <>
-struct PipeCfg<4, true> {
-  static constexpr int EPB = ESDG_PIPE4_EPB32, MINB = ESDG_PIPE4_MINB32;
-};
-// the pipelined kernels' Shape (the mixed one carries the background fields)
-template <int N, bool MIXED>
-using PipeShape = Shape<N, MIXED, MIXED, PipeCfg<N, MIXED>::EPB>;
+// the pipelined kernel's Shape
+template <int N>
+using PipeShape = Shape<N, true, true>;
 
 // The tile with index t: (member, first element, elements).  TABLE: from the
 // work table (EPB elements, fewer at a member's end).  SINGLE: EPB-element
@@ -100,23 +71,6 @@ struct PipeCtl {
   unsigned long long bars[2];  // [0] RAW of the next tile, [1] CUR of this tile
   int4 info[2];  // (member, first element, elements)
   EsdgMember desc[TABLE ? 2 : 1];
-};
-
-template <int N, int MODE>
-struct Pipe64 {
-  using SH = PipeShape<N, false>;
-  static constexpr int P = SH::NP * SH::EPB;  // nodes per tile
-  static constexpr int even(int x) { return (x + 1) & ~1; }
-  // offsets in doubles, all even (16-byte aligned); each copy target holds
-  // four extra doubles for the aligned span around its block
-  static constexpr int RAW_Q = 0;                            // [el][5][NP]   next tile's q
-  static constexpr int RAW_G = even(RAW_Q + 5 * P + 4);      // [el][11][NP]  next tile's geometry
-  static constexpr int S0 = even(RAW_G + ESDG_NVGEO * P + 4);  // [el][18][NP] primitives, Ja/2; exchange
-  static constexpr int EPI = even(S0 + SH::NF * P);          // [el][6][NP]   q and 1/J of this tile
-  static constexpr int DQ = even(EPI + 6 * P);               // [el][5][NP]   dq of this tile
-  static constexpr int TOTAL = MODE ? DQ + 5 * P + 4 : DQ;
-  static constexpr size_t SMEM = sizeof(double) * (size_t)TOTAL;
-  static_assert(SH::NF == 18, "FP64 node fields");
 };
 
 // One block copy of a tile: n elements (4 or 8 bytes) at src, an array that
@@ -218,237 +172,10 @@ __device__ __forceinline__ void pipe_issue(int tid, const BlockCopy (&bl)[MAXB],
                  : "memory");
 }
 
-template <int N, int MODE, bool TABLE>
-__global__ void __launch_bounds__(PipeShape<N, false>::THREADS, PipeCfg<N, false>::MINB)
-    k_volume_pipe64(const EsdgMember one, const EsdgMember* __restrict__ members,
-                    const int2* __restrict__ tiles, const int* __restrict__ ntiles_d, int ntiles_1,
-                    EsdgLGL L, double rkA, double rkB, unsigned phantom, int t1, int s1) {
-  static_assert(!TABLE || MODE == 1, "the batched kernel applies an RK stage");
-  using SH = PipeShape<N, false>;
-  using PP = Pipe64<N, MODE>;
-  constexpr int Nq = SH::Nq, NP = SH::NP, NPEN = SH::NPEN, EPB = SH::EPB, NF = SH::NF;
-  constexpr int T = SH::THREADS;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ __align__(16) PipeCtl<TABLE> ctl;
-  double* sm = reinterpret_cast<double*>(smraw);
-  const int tid = threadIdx.x;
-  const int ntiles = TABLE ? *ntiles_d : ntiles_1;
-
-  using ISS = Issuers<T, SH::PENCILS>;
-  // the next tile as seen by the issuing lanes (fetched early: in TABLE mode
-  // these are global loads whose latency the prologue hides)
-  struct Next {
-    int4 tr;  // (member, first element, elements)
-    int E;
-    const double* q;
-    const double* vg;
-    const EsdgMember* Mg;
-  };
-  auto fetch = [&](int t) {
-    Next x;
-    const int m = TABLE ? tiles[t].x : 0;
-    x.Mg = TABLE ? members + m : &ctl.desc[0];
-    x.E = x.Mg->g.E;
-    x.tr = pipe_tile<TABLE, EPB>(tiles, t, t1, s1, x.E);
-    x.q = x.Mg->a.q_in;
-    x.vg = reinterpret_cast<const double*>(x.Mg->a.vgeo);
-    return x;
-  };
-  // issuing lanes: the next tile's (member, e0), descriptor and RAW blocks into slot s
-  auto issue_next = [&](const Next& x, int s, unsigned ph = 0) {
-    if (tid == ISS::FIRST) ctl.info[s] = x.tr;
-    const int e0 = x.tr.y, ne = x.tr.z;
-    const BlockCopy bl[2] = {
-        {sm + PP::RAW_Q, x.q + (size_t)e0 * 5 * NP, x.q + (size_t)x.E * 5 * NP, ne * 5 * NP, 8},
-        {sm + PP::RAW_G, x.vg + (size_t)e0 * ESDG_NVGEO * NP, x.vg + (size_t)x.E * ESDG_NVGEO * NP,
-         ne * ESDG_NVGEO * NP, 8}};
-    if constexpr (TABLE)
-      pipe_issue<ISS>(tid, bl, 2, &ctl.bars[0], (unsigned)sizeof(EsdgMember), x.Mg, &ctl.desc[s], ph);
-    else
-      pipe_issue<ISS>(tid, bl, 2, &ctl.bars[0], 0, nullptr, nullptr, ph);
-  };
-
-  if (tid == 0) {
-    esdg_mbar_init(&ctl.bars[0], 1);
-    esdg_mbar_init(&ctl.bars[1], 1);
-    esdg_fence_mbar_init();
-    if constexpr (!TABLE) ctl.desc[0] = one;
-  }
-  __syncthreads();
-  if (ISS::is(tid) && (int)blockIdx.x < ntiles) issue_next(fetch(blockIdx.x), 0, phantom);
-  unsigned ph_raw = 0, ph_cur = 0;
-  int slot = 0;
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, slot ^= 1) {
-    esdg_cp_async_wait_all();  // this lane's tail copies
-    const bool ok = esdg_mbar_wait(&ctl.bars[0], ph_raw, ESDG_WAIT_LIMIT);
-    ph_raw ^= 1u;
-    if (__syncthreads_or(!ok)) {
-      if (tid == 0) atomicExch(&g_esdg_vol_timeout, 1);
-      return;
-    }
-    const EsdgMember& M = ctl.desc[TABLE ? slot : 0];
-    const EsdgGrid& g = M.g;
-    const EsdgPhys& P = M.P;
-    const EsdgVolArgs& a = M.a;
-    const int E = g.E, e0 = ctl.info[slot].y, ne = ctl.info[slot].z;
-    const int next = tile + (int)gridDim.x;
-    // issuing lanes: this tile's dq (CUR) now, the next tile's location early
-    Next nx;
-    if (ISS::is(tid)) {
-      if constexpr (MODE != 0) {
-        const double* dqg = reinterpret_cast<const double*>(a.dq);
-        const BlockCopy cb[1] = {{sm + PP::DQ, dqg + (size_t)e0 * 5 * NP, dqg + (size_t)E * 5 * NP,
-                                  ne * 5 * NP, 8}};
-        pipe_issue<ISS>(tid, cb, 1, &ctl.bars[1]);
-      }
-      if (TABLE && next < ntiles) nx = fetch(next);  // global loads: early
-    }
-    // ---- prologue: RAW -> primitives, Ja/2 (S) and q, 1/J (EPI) -----------
-    {
-      const double* vg = reinterpret_cast<const double*>(a.vgeo);
-      const double* qr0 = sm + PP::RAW_Q + esdg_block_shift(a.q_in + (size_t)e0 * 5 * NP);
-      const double* gr0 = sm + PP::RAW_G + esdg_block_shift(vg + (size_t)e0 * ESDG_NVGEO * NP);
-      const double gm1 = P.gamma - 1.0;
-      for (int idx = tid; idx < EPB * NP; idx += T) {
-        const int el2 = idx / NP, n = idx - el2 * NP;
-        double* S = sm + PP::S0 + (size_t)el2 * NF * NP;
-        if (el2 < ne) {
-          const double* qr = qr0 + (size_t)el2 * 5 * NP;
-          const double* gr = gr0 + (size_t)el2 * ESDG_NVGEO * NP;
-          double* X = sm + PP::EPI + (size_t)el2 * 6 * NP;
-          const double q0 = qr[n], q1 = qr[NP + n], q2 = qr[2 * NP + n], q3 = qr[3 * NP + n],
-                       q4 = qr[4 * NP + n];
-          prims64<NP>(q0, q1, q2, q3, q4, gr[10 * NP + n], gm1, S, n);
-#pragma unroll
-          for (int k = 0; k < 9; k++) S[(SH::F_NH + k) * NP + n] = gr[k * NP + n];
-          X[n] = q0;
-          X[NP + n] = q1;
-          X[2 * NP + n] = q2;
-          X[3 * NP + n] = q3;
-          X[4 * NP + n] = q4;
-          // 1/J, times dt for a stage update (the epilogue's scale)
-          X[5 * NP + n] = MODE != 0 ? gr[9 * NP + n] * a.dt : gr[9 * NP + n];
-        } else {  // padding element: any valid state, results are discarded
-          S[0 * NP + n] = 0.25;
-          S[1 * NP + n] = 0.5;
-          S[2 * NP + n] = 1.0;
-          for (int k = 3; k < NF; k++) S[k * NP + n] = 0.0;
-        }
-      }
-    }
-    __syncthreads();  // RAW consumed
-
-    int need_logs = 0;
-    for (int idx = tid; idx < EPB * NP; idx += T) {
-      const int el2 = idx / NP, n = idx - el2 * NP;
-      if (out_of_series64<NP>(sm + PP::S0 + (size_t)el2 * NF * NP, n)) need_logs = 1;
-    }
-    need_logs = __syncthreads_or(need_logs);
-    if (need_logs) {
-      for (int idx = tid; idx < EPB * NP; idx += T) {
-        const int el2 = idx / NP, n = idx - el2 * NP;
-        double* S = sm + PP::S0 + (size_t)el2 * NF * NP;
-        S[SH::F_LR * NP + n] = log(4.0 * S[n]);
-        S[SH::F_LB * NP + n] = log(2.0 * S[NP + n]);
-      }
-      __syncthreads();
-    }
-    // the copies for this tile's epilogue and the next tile
-    if (ISS::is(tid) && next < ntiles) issue_next(TABLE ? nx : fetch(next), slot ^ 1);
-
-    // ---- pair pass: this thread's pencil (index arithmetic redone per tile
-    // rather than held in registers across the pair pass) -------------------
-    const bool active = tid < SH::PENCILS;
-    const int el = active ? tid / (3 * NPEN) : 0;
-    const int rr = tid - el * 3 * NPEN;
-    const int d = active ? rr / NPEN : 0;
-    const int pen = rr - d * NPEN;
-    const int ps = pen % Nq, pt = pen / Nq;
-    const int stride = (d == 0) ? 1 : ((d == 1) ? Nq : Nq * Nq);
-    const int base = (d == 0) ? Nq * (ps + Nq * pt) : ((d == 1) ? (ps + Nq * Nq * pt) : (ps + Nq * pt));
-    const int e = e0 + el;
-    double acc[Nq][5];
-#pragma unroll
-    for (int i = 0; i < Nq; i++)
-#pragma unroll
-      for (int v = 0; v < 5; v++) acc[i][v] = 0.0;
-    if (active && el < ne) {
-      face_lift<true, N, double>(g, a, e, d, ps + Nq * pt, acc);
-      const double* S = sm + PP::S0 + (size_t)el * NF * NP;
-      if (need_logs)
-        pencil_pass<N, false, true, false>(S, d, base, stride, L, ce_series(0.5 * P.igm1), acc);
-      else
-        pencil_pass<N, false, false, false>(S, d, base, stride, L, ce_series(0.5 * P.igm1), acc);
-    }
-    __syncthreads();
-    if (active && el < ne) {
-      double* S = sm + PP::S0 + (size_t)el * NF * NP;
-#pragma unroll
-      for (int i = 0; i < Nq; i++)
-#pragma unroll
-        for (int v = 0; v < 5; v++) S[(d * 5 + v) * NP + base + i * stride] = acc[i][v];
-    }
-    if constexpr (MODE != 0) {
-      esdg_cp_async_wait_all();
-      const bool okd = esdg_mbar_wait(&ctl.bars[1], ph_cur, ESDG_WAIT_LIMIT);  // this tile's dq
-      ph_cur ^= 1u;
-      if (__syncthreads_or(!okd)) {
-        if (tid == 0) {
-          atomicExch(&g_esdg_vol_timeout, 1);
-          pipe_drain(&ctl.bars[0], ph_raw, next < ntiles);
-        }
-        return;
-      }
-    } else {
-      __syncthreads();
-    }
-
-    // ---- epilogue: one thread per (node, variable) (eight full rounds instead
-    // of one and a partial one per node) ---------------------------------------
-    const double* D0 = sm + PP::DQ + esdg_block_shift(reinterpret_cast<const double*>(a.dq) + (size_t)e0 * 5 * NP);
-    // descriptor fields in registers (the stores below would force reloads)
-    const double dt = a.dt;
-    const EsdgPhys Pl = P;
-    const bool rot = (Pl.f0 != 0.0) || (Pl.beta != 0.0);
-    const double* xg = a.x;
-    double* const dqp = reinterpret_cast<double*>(a.dq);
-    double* const qio = a.q_io;
-    double* const rhsp = a.rhs;
-    int* const status = a.status;
-    bool bad = false;
-    for (int idx = tid; idx < 5 * EPB * NP; idx += T) {
-      const int v = idx / (EPB * NP), rem = idx - v * (EPB * NP);
-      const int el2 = rem / NP, n = rem - el2 * NP, e2 = e0 + el2;
-      if (el2 >= ne) continue;
-      const double* S = sm + PP::S0 + (size_t)el2 * NF * NP;
-      const double* X = sm + PP::EPI + (size_t)el2 * 6 * NP;
-      double r = -X[5 * NP + n] * (S[v * NP + n] + S[(5 + v) * NP + n] + S[(10 + v) * NP + n]);
-      if (rot && (v == 1 || v == 2)) {
-        const double y = xg[((size_t)e2 * 3 + 1) * NP + n];
-        double f = Pl.f0 + Pl.beta * (y - Pl.y0);
-        if constexpr (MODE != 0) f *= dt;
-        r = v == 1 ? fma(f, X[2 * NP + n], r) : fma(-f, X[NP + n], r);
-      }
-      const size_t qv = ((size_t)e2 * 5 + v) * NP + n;
-      if constexpr (MODE == 0) {
-        rhsp[qv] = r;
-      } else {
-        // first stage (A = 0): the register is not read (see stage32)
-        const double dv = rkA == 0.0 ? r : fma(rkA, D0[((size_t)el2 * 5 + v) * NP + n], r);
-        dqp[qv] = dv;
-        const double qn = fma(rkB, dv, X[v * NP + n]);
-        qio[qv] = qn;
-        bad |= esdg_bad_state(qn, v == 0);
-      }
-    }
-    if (MODE != 0 && bad && status) *status = 1;
-  }
-}
-
 // ---- pipelined persistent mixed-precision kernel (with a background) ------
 template <int N, int MODE>
 struct Pipe32 {
-  using SH = PipeShape<N, true>;
+  using SH = PipeShape<N>;
   static constexpr int NP = SH::NP, EPB = SH::EPB, P = NP * EPB;
   static constexpr int up16(int b) { return (b + 15) & ~15; }
   // byte offsets, 16-byte aligned; copy targets hold 32 extra bytes (the
@@ -467,12 +194,12 @@ struct Pipe32 {
 };
 
 template <int N, int MODE, bool TABLE>
-__global__ void __launch_bounds__(PipeShape<N, true>::THREADS, PipeCfg<N, true>::MINB)
+__global__ void __launch_bounds__(PipeShape<N>::THREADS, 1)
     k_volume_pipe32(const EsdgMember one, const EsdgMember* __restrict__ members,
                     const int2* __restrict__ tiles, const int* __restrict__ ntiles_d, int ntiles_1,
                     EsdgLGL L, double rkA, double rkB, unsigned phantom, int t1, int s1) {
   static_assert(!TABLE || MODE == 1, "the batched kernel applies an RK stage");
-  using SH = PipeShape<N, true>;
+  using SH = PipeShape<N>;
   using PP = Pipe32<N, MODE>;
   constexpr int Nq = SH::Nq, NP = SH::NP, NPEN = SH::NPEN, EPB = SH::EPB, NF = SH::NF;
   constexpr int T = SH::THREADS;
@@ -686,9 +413,9 @@ __global__ void __launch_bounds__(PipeShape<N, true>::THREADS, PipeCfg<N, true>:
       const float* S = sm + (size_t)el * NF * NP;
       const float ce = esdg_d2f(0.5 * P.igm1);
       if (need_logs)
-        pencil_pass<N, true, true, true>(S, d, base, stride, L, ce, acc);
+        pencil_pass<N, true, true>(S, d, base, stride, L, ce, acc);
       else
-        pencil_pass<N, true, false, true>(S, d, base, stride, L, ce, acc);
+        pencil_pass<N, false, true>(S, d, base, stride, L, ce, acc);
       const float phi0 = phi0s[el];
 #pragma unroll
       for (int i = 0; i < Nq; i++) acc[i][4] = fmaf(phi0, acc[i][0], acc[i][4]);
@@ -820,25 +547,9 @@ inline EsdgMember pipe_member(const EsdgGrid& g, const EsdgPhys& P, const EsdgVo
 }
 
 template <int N, int MODE>
-cudaError_t launch_pipe64(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL& L,
-                          const EsdgVolArgs& a, cudaStream_t s) {
-  using SH = PipeShape<N, false>;
-  constexpr auto k = k_volume_pipe64<N, MODE, false>;
-  const int cap = pipe_grid_cap<k>(SH::THREADS, Pipe64<N, MODE>::SMEM);
-  if (cap < 0) return cudaErrorInvalidConfiguration;
-  int ntiles, grid, t1, s1;
-  pipe_split(g.E, SH::EPB, cap, ntiles, grid, t1, s1);
-  if (ntiles == 0) return cudaSuccess;
-  k<<<grid, SH::THREADS, Pipe64<N, MODE>::SMEM, s>>>(pipe_member(g, P, a), nullptr, nullptr, nullptr,
-                                                     ntiles, L, a.rkA, a.rkB, esdg_take_phantom(),
-                                                     t1, s1);
-  return cudaGetLastError();
-}
-
-template <int N, int MODE>
 cudaError_t launch_pipe32(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL& L,
                           const EsdgVolArgs& a, cudaStream_t s) {
-  using SH = PipeShape<N, true>;
+  using SH = PipeShape<N>;
   constexpr auto k = k_volume_pipe32<N, MODE, false>;
   const int cap = pipe_grid_cap<k>(SH::THREADS, Pipe32<N, MODE>::SMEM);
   if (cap < 0) return cudaErrorInvalidConfiguration;
@@ -852,16 +563,13 @@ cudaError_t launch_pipe32(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL& L
 }
 
 // batched (TABLE) launches; what: 0 launch (0 / -1), 1 elements per tile, 2 CTAs per SM
-template <int N, bool MIXED>
+template <int N>
 int pipe_batch(int what, const EsdgMember* members, const int2* tiles, const int* ntiles, int grid,
                const EsdgLGL& L, double A, double B, cudaStream_t s) {
-  using SH = PipeShape<N, MIXED>;
-  constexpr size_t SMEM = MIXED ? Pipe32<N, 1>::SMEM : Pipe64<N, 1>::SMEM;
+  using SH = PipeShape<N>;
+  constexpr size_t SMEM = Pipe32<N, 1>::SMEM;
   if (what == 1) return SH::EPB;
-  auto k = [] {
-    if constexpr (MIXED) return k_volume_pipe32<N, 1, true>;
-    else return k_volume_pipe64<N, 1, true>;
-  }();
+  constexpr auto k = k_volume_pipe32<N, 1, true>;
   if (what == 2) {
     int nb = 0;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM) != cudaSuccess ||

@@ -1,4 +1,4 @@
-// volume_tile.cuh -- the per-tile volume kernel: one CTA per tile of EPB
+// volume_tile.cuh -- the mixed path's per-tile volume kernel: one CTA per tile of EPB
 // elements (k_volume), its persistent batched form over a device work table
 // (k_volume_batch), and their launchers.  Used for the mixed path without a
 // background or with a moving one, for tiles whose pipelined form exceeds
@@ -10,10 +10,10 @@ namespace esdg_vol {
 
 // One tile: elements e0 .. e0 + EPB - 1 of one mesh, processed by a CTA of
 // SH::THREADS threads with SH::SMEM bytes of shared memory at smraw.
-template <int N, bool MIXED, int MODE, int BG, int EPB_ = 0>
+template <int N, int MODE, int BG, int EPB_ = 0>
 __device__ __forceinline__ void volume_tile(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL& L,
                                             const EsdgVolArgs& a, int e0, unsigned char* smraw) {
-  using SH = Shape<N, MIXED, BG, EPB_>;
+  using SH = Shape<N, true, BG, EPB_>;
   using R = typename SH::R;
   constexpr int Nq = SH::Nq, NP = SH::NP, NPEN = SH::NPEN, EPB = SH::EPB, NF = SH::NF;
   constexpr int T = SH::THREADS;
@@ -33,37 +33,33 @@ __device__ __forceinline__ void volume_tile(const EsdgGrid& g, const EsdgPhys& P
       const double q0 = qe[n], q1 = qe[NP + n], q2 = qe[2 * NP + n], q3 = qe[3 * NP + n],
                    q4 = qe[4 * NP + n];
       const double phi = a.vgeo64[((size_t)e * ESDG_NVGEO + 10) * NP + n];
-      if constexpr (MIXED) {
-        const float phh = vg[((size_t)e * ESDG_NVGEO + 10) * NP + n];
-        if constexpr (BG == 2) {
-          const double* bq = a.bgq + (size_t)e * 5 * NP + n;
-          const float* bpe = a.bgp + (size_t)e * 4 * NP + n;
-          const float* bu = a.bgu + (size_t)e * 3 * NP + n;
-          const Prim32m o = prims32bgm(q0, q1, q2, q3, q4, phi, phh, gm1f, bq[0], bq[NP],
-                                       bq[2 * NP], bq[3 * NP], bq[4 * NP], bpe[0], bpe[NP],
-                                       bpe[2 * NP], bpe[3 * NP], bu[0], bu[NP], bu[2 * NP]);
+      const float phh = vg[((size_t)e * ESDG_NVGEO + 10) * NP + n];
+      if constexpr (BG == 2) {
+        const double* bq = a.bgq + (size_t)e * 5 * NP + n;
+        const float* bpe = a.bgp + (size_t)e * 4 * NP + n;
+        const float* bu = a.bgu + (size_t)e * 3 * NP + n;
+        const Prim32m o = prims32bgm(q0, q1, q2, q3, q4, phi, phh, gm1f, bq[0], bq[NP],
+                                     bq[2 * NP], bq[3 * NP], bq[4 * NP], bpe[0], bpe[NP],
+                                     bpe[2 * NP], bpe[3 * NP], bu[0], bu[NP], bu[2 * NP]);
 #pragma unroll
-          for (int k = 0; k < 7; k++) {
-            S[k * NP + n] = o.s[k];
-            S[(SH::F_BG + k) * NP + n] = o.bgf[k];
-          }
+        for (int k = 0; k < 7; k++) {
+          S[k * NP + n] = o.s[k];
+          S[(SH::F_BG + k) * NP + n] = o.bgf[k];
+        }
 #pragma unroll
-          for (int k = 0; k < 3; k++) S[(SH::F_BG + 7 + k) * NP + n] = o.up[k];
-        } else if constexpr (BG) {
-          const double* bge = a.bg + (size_t)e * 3 * NP;
-          const float* bpe = a.bgp + (size_t)e * 4 * NP;
-          const Prim32 o = prims32bg(q0, q1, q2, q3, q4, phi, phh, gm1f, bge[n], bge[NP + n],
-                                     bpe[n], bpe[NP + n], bpe[2 * NP + n], bpe[3 * NP + n]);
+        for (int k = 0; k < 3; k++) S[(SH::F_BG + 7 + k) * NP + n] = o.up[k];
+      } else if constexpr (BG) {
+        const double* bge = a.bg + (size_t)e * 3 * NP;
+        const float* bpe = a.bgp + (size_t)e * 4 * NP;
+        const Prim32 o = prims32bg(q0, q1, q2, q3, q4, phi, phh, gm1f, bge[n], bge[NP + n],
+                                   bpe[n], bpe[NP + n], bpe[2 * NP + n], bpe[3 * NP + n]);
 #pragma unroll
-          for (int k = 0; k < 7; k++) {
-            S[k * NP + n] = o.s[k];
-            S[(SH::F_BG + k) * NP + n] = o.bgf[k];
-          }
-        } else {
-          prims32<NP>(q0, q1, q2, q3, q4, phi, phh, gm1, S, n);
+        for (int k = 0; k < 7; k++) {
+          S[k * NP + n] = o.s[k];
+          S[(SH::F_BG + k) * NP + n] = o.bgf[k];
         }
       } else {
-        prims64<NP>(q0, q1, q2, q3, q4, phi, gm1, S, n);
+        prims32<NP>(q0, q1, q2, q3, q4, phi, phh, gm1, S, n);
       }
 #pragma unroll
       for (int k = 0; k < 9; k++)
@@ -76,31 +72,14 @@ __device__ __forceinline__ void volume_tile(const EsdgGrid& g, const EsdgPhys& P
     }
   }
   __syncthreads();
-  if constexpr (!MIXED) {
-    for (int idx = threadIdx.x; idx < EPB * NP; idx += T) {
-      const int el = idx / NP, n = idx - el * NP;
-      if (out_of_series64<NP>(sm + (size_t)el * NF * NP, n)) need_logs = 1;
-    }
-    need_logs = __syncthreads_or(need_logs);
-    if (need_logs) {
-      for (int idx = threadIdx.x; idx < EPB * NP; idx += T) {
-        const int el = idx / NP, n = idx - el * NP;
-        R* S = sm + (size_t)el * NF * NP;
-        S[SH::F_LR * NP + n] = log(4.0 * S[n]);
-        S[SH::F_LB * NP + n] = log(2.0 * S[NP + n]);
-      }
-      __syncthreads();
-    }
-  } else {
-    for (int idx = threadIdx.x; idx < EPB * NP; idx += T) {
-      const int el = idx / NP, n = idx - el * NP;
-      const R* S = sm + (size_t)el * NF * NP;
-      const float r0 = S[0], rn = S[n], b0 = S[NP], bn = S[NP + n];
-      // |f| < 0.14 keeps u < ESDG_LOG_EPS32 for every pair
-      if (fabsf(rn - r0) > 0.13f * r0 || fabsf(bn - b0) > 0.13f * b0) need_logs = 1;
-    }
-    need_logs = __syncthreads_or(need_logs);
+  for (int idx = threadIdx.x; idx < EPB * NP; idx += T) {
+    const int el = idx / NP, n = idx - el * NP;
+    const R* S = sm + (size_t)el * NF * NP;
+    const float r0 = S[0], rn = S[n], b0 = S[NP], bn = S[NP + n];
+    // |f| < 0.14 keeps u < ESDG_LOG_EPS32 for every pair
+    if (fabsf(rn - r0) > 0.13f * r0 || fabsf(bn - b0) > 0.13f * b0) need_logs = 1;
   }
+  need_logs = __syncthreads_or(need_logs);
 
   // ---- pair pass: one pencil per thread ---------------------------------
   const int tid = threadIdx.x;
@@ -118,32 +97,21 @@ __device__ __forceinline__ void volume_tile(const EsdgGrid& g, const EsdgPhys& P
   for (int i = 0; i < Nq; i++)
 #pragma unroll
     for (int v = 0; v < 5; v++) acc[i][v] = (R)0;
-  if constexpr (!MIXED)
-    if (active && e < E) face_lift<true, N, R>(g, a, e, d, s + Nq * t, acc);
   if (active && e < E) {
-    // mixed: the face terms and the element's reference geopotential are
-    // fetched ahead of the pair pass and applied after it
-    FaceTerms<R> ft{};
-    R phi0 = (R)0;
-    if constexpr (MIXED) {
-      ft = face_fetch<N, R>(g, a, e, d, s + Nq * t);
-      phi0 = esdg_d2f(a.vgeo64[((size_t)e * ESDG_NVGEO + 10) * NP]);
-    }
+    // the face terms and the element's reference geopotential are fetched
+    // ahead of the pair pass and applied after it
+    const FaceTerms<R> ft = face_fetch<N, R>(g, a, e, d, s + Nq * t);
+    const R phi0 = esdg_d2f(a.vgeo64[((size_t)e * ESDG_NVGEO + 10) * NP]);
     const R* S = sm + (size_t)el * NF * NP;
-    const auto ce = [&] {
-      if constexpr (MIXED) return esdg_d2f(0.5 * P.igm1);
-      else return ce_series(0.5 * P.igm1);
-    }();
+    const float ce = esdg_d2f(0.5 * P.igm1);
     if (need_logs)
-      pencil_pass<N, MIXED, true, BG>(S, d, base, stride, L, ce, acc);
+      pencil_pass<N, true, BG>(S, d, base, stride, L, ce, acc);
     else
-      pencil_pass<N, MIXED, false, BG>(S, d, base, stride, L, ce, acc);
-    if constexpr (MIXED) {
-      // restore the element's reference geopotential in the energy flux
+      pencil_pass<N, false, BG>(S, d, base, stride, L, ce, acc);
+    // restore the element's reference geopotential in the energy flux
 #pragma unroll
-      for (int i = 0; i < Nq; i++) acc[i][4] = fmaf(phi0, acc[i][0], acc[i][4]);
-      face_add<N, R>(ft, acc);
-    }
+    for (int i = 0; i < Nq; i++) acc[i][4] = fmaf(phi0, acc[i][0], acc[i][4]);
+    face_add<N, R>(ft, acc);
   }
   __syncthreads();
   if (active && e < E) {
@@ -162,7 +130,7 @@ __device__ __forceinline__ void volume_tile(const EsdgGrid& g, const EsdgPhys& P
     const int el2 = idx / NP, n = idx - el2 * NP, e2 = e0 + el2;
     if (e2 >= E) continue;
     const R* S = sm + (size_t)el2 * NF * NP;
-    if constexpr (MIXED && MODE != 0) {
+    if constexpr (MODE != 0) {
       const float iJf = vg[((size_t)e2 * ESDG_NVGEO + 9) * NP + n];
       float r32[5];
 #pragma unroll
@@ -176,16 +144,12 @@ __device__ __forceinline__ void volume_tile(const EsdgGrid& g, const EsdgPhys& P
                              a.rkB, a.dt, BG == 2 ? a.bgq + qb : nullptr);
       continue;
     }
-    // FP64 stage update: dt is folded into the -1/J scale (r then holds dt rhs)
-    constexpr bool DT_IN_R = !MIXED && MODE != 0;
-    R iJ = vg[((size_t)e2 * ESDG_NVGEO + 9) * NP + n];
-    if constexpr (DT_IN_R) iJ *= a.dt;
+    const R iJ = vg[((size_t)e2 * ESDG_NVGEO + 9) * NP + n];
     double r[5];
 #pragma unroll
     for (int v = 0; v < 5; v++) {
       const R rv = -iJ * (S[v * NP + n] + S[(5 + v) * NP + n] + S[(10 + v) * NP + n]);
-      if constexpr (MIXED) r[v] = esdg_f2d(rv);
-      else r[v] = rv;
+      r[v] = esdg_f2d(rv);
     }
     const size_t qb = (size_t)e2 * 5 * NP + n;
     if constexpr (BG == 2) {  // the moving background's own right-hand side
@@ -198,50 +162,32 @@ __device__ __forceinline__ void volume_tile(const EsdgGrid& g, const EsdgPhys& P
     }
     if (rotating) {
       const double y = a.x[((size_t)e2 * 3 + 1) * NP + n];
-      double f = P.f0 + P.beta * (y - P.y0);
-      if constexpr (DT_IN_R) f *= a.dt;
+      const double f = P.f0 + P.beta * (y - P.y0);
       // with a moving background its Coriolis force is part of its rhs
       const double my = BG == 2 ? a.q_in[qb + 2 * NP] - a.bgq[qb + 2 * NP] : a.q_in[qb + 2 * NP];
       const double mx = BG == 2 ? a.q_in[qb + NP] - a.bgq[qb + NP] : a.q_in[qb + NP];
       r[1] = fma(f, my, r[1]);
       r[2] = fma(-f, mx, r[2]);
     }
-    if constexpr (MODE == 0) {
 #pragma unroll
-      for (int v = 0; v < 5; v++) a.rhs[qb + (size_t)v * NP] = r[v];
-    } else {
-      if constexpr (MIXED) {
-        // handled above
-      } else {
-        double* dq = reinterpret_cast<double*>(a.dq);
-#pragma unroll
-        for (int v = 0; v < 5; v++) {
-          // first stage (A = 0): the register is not read (see stage32)
-          const double dv = a.rkA == 0.0 ? r[v] : fma(a.rkA, dq[qb + (size_t)v * NP], r[v]);
-          dq[qb + (size_t)v * NP] = dv;
-          const double qn = fma(a.rkB, dv, a.q_in[qb + (size_t)v * NP]);
-          a.q_io[qb + (size_t)v * NP] = qn;
-          bad |= esdg_bad_state(qn, v == 0);
-        }
-      }
-    }
+    for (int v = 0; v < 5; v++) a.rhs[qb + (size_t)v * NP] = r[v];
   }
   if (MODE != 0 && bad && a.status) *a.status = 1;
 }
 
-template <int N, bool MIXED, int MODE, int BG>
-__global__ void __launch_bounds__(Shape<N, MIXED, BG>::THREADS)
+template <int N, int MODE, int BG>
+__global__ void __launch_bounds__(Shape<N, true, BG>::THREADS)
     k_volume(EsdgGrid g, EsdgPhys P, EsdgLGL L, EsdgVolArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  volume_tile<N, MIXED, MODE, BG>(g, P, L, a, blockIdx.x * Shape<N, MIXED, BG>::EPB, smraw);
+  volume_tile<N, MODE, BG>(g, P, L, a, blockIdx.x * Shape<N, true, BG>::EPB, smraw);
 }
 
 // Persistent batched volume kernel: CTAs stride over a device work table of
 // (member, first element) tiles of meshes with the same N and precision and
 // apply one LSRK stage to each (dt per member, stage coefficients per launch).
 // The member descriptor of the current tile is staged in shared memory.
-template <int N, bool MIXED, bool BG, int EPB_>
-__global__ void __launch_bounds__(Shape<N, MIXED, BG, EPB_>::THREADS)
+template <int N, bool BG, int EPB_>
+__global__ void __launch_bounds__(Shape<N, true, BG, EPB_>::THREADS)
     k_volume_batch(const EsdgMember* __restrict__ members, const int2* __restrict__ tiles,
                    const int* __restrict__ ntiles, EsdgLGL L, double rkA, double rkB) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -261,18 +207,18 @@ __global__ void __launch_bounds__(Shape<N, MIXED, BG, EPB_>::THREADS)
       mb.a.rkB = rkB;
     }
     __syncthreads();
-    volume_tile<N, MIXED, 1, BG, EPB_>(mb.g, mb.P, L, mb.a, tile.y, smraw);
+    volume_tile<N, 1, BG, EPB_>(mb.g, mb.P, L, mb.a, tile.y, smraw);
     __syncthreads();
   }
 }
 
-template <int N, bool MIXED, int MODE, int BG>
+template <int N, int MODE, int BG>
 cudaError_t launch_one(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL& L,
                        const EsdgVolArgs& a, cudaStream_t s) {
-  using SH = Shape<N, MIXED, BG>;
+  using SH = Shape<N, true, BG>;
   static bool configured = false;  // one-time attribute set per instantiation
   if (!configured) {
-    cudaError_t err = cudaFuncSetAttribute(k_volume<N, MIXED, MODE, BG>,
+    cudaError_t err = cudaFuncSetAttribute(k_volume<N, MODE, BG>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)SH::SMEM);
     if (err != cudaSuccess) return err;
@@ -280,34 +226,34 @@ cudaError_t launch_one(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL& L,
   }
   const unsigned blocks = (unsigned)((g.E + SH::EPB - 1) / SH::EPB);
   if (blocks == 0) return cudaSuccess;
-  k_volume<N, MIXED, MODE, BG><<<blocks, SH::THREADS, SH::SMEM, s>>>(g, P, L, a);
+  k_volume<N, MODE, BG><<<blocks, SH::THREADS, SH::SMEM, s>>>(g, P, L, a);
   return cudaGetLastError();
 }
 
-template <int N, bool MIXED, bool BG, int EPB_>
+template <int N, bool BG, int EPB_>
 cudaError_t launch_batch_one(const EsdgMember* members, const int2* tiles, const int* ntiles,
                              int grid, const EsdgLGL& L, double A, double B, cudaStream_t s) {
-  using SH = Shape<N, MIXED, BG, EPB_>;
+  using SH = Shape<N, true, BG, EPB_>;
   static bool configured = false;
   if (!configured) {
-    cudaError_t err = cudaFuncSetAttribute(k_volume_batch<N, MIXED, BG, EPB_>,
+    cudaError_t err = cudaFuncSetAttribute(k_volume_batch<N, BG, EPB_>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)SH::SMEM);
     if (err != cudaSuccess) return err;
     configured = true;
   }
-  k_volume_batch<N, MIXED, BG, EPB_><<<grid, SH::THREADS, SH::SMEM, s>>>(members, tiles, ntiles, L,
+  k_volume_batch<N, BG, EPB_><<<grid, SH::THREADS, SH::SMEM, s>>>(members, tiles, ntiles, L,
                                                                           A, B);
   return cudaGetLastError();
 }
 
-template <int N, bool MIXED, bool BG, int EPB_>
+template <int N, bool BG, int EPB_>
 int batch_occupancy() {
-  using SH = Shape<N, MIXED, BG, EPB_>;
+  using SH = Shape<N, true, BG, EPB_>;
   int nb = 0;
-  cudaFuncSetAttribute(k_volume_batch<N, MIXED, BG, EPB_>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_volume_batch<N, BG, EPB_>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)SH::SMEM);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_volume_batch<N, MIXED, BG, EPB_>,
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_volume_batch<N, BG, EPB_>,
                                                     SH::THREADS, SH::SMEM) != cudaSuccess) {
     cudaGetLastError();
     return 1;

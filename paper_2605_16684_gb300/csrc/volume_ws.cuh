@@ -430,9 +430,9 @@ __global__ void __launch_bounds__(Ws32<N, MODE>::T, 1)
         const FaceTerms<float> ft = face_fetch<N, float>(g, a, e0 + el, d, ps + Nq * pt);
         const float* S = Sb + (size_t)el * NF * NP;
         if (need_logs)
-          pencil_pass<N, true, true, true>(S, d, base, stride, L, ce, acc);
+          pencil_pass<N, true, true>(S, d, base, stride, L, ce, acc);
         else
-          pencil_pass<N, true, false, true>(S, d, base, stride, L, ce, acc);
+          pencil_pass<N, false, true>(S, d, base, stride, L, ce, acc);
         const float phi0 = c.phi0[b][el];
 #pragma unroll
         for (int i = 0; i < Nq; i++) acc[i][4] = fmaf(phi0, acc[i][0], acc[i][4]);
