@@ -195,6 +195,7 @@ EsdgVolArgs vol_args(es_dg_t* h, const double* q_in, double* rhs_out) {
   a.rkB = 0.0;
   a.dt = 0.0;
   a.status = h->status;
+  a.share = 1;
   return a;
 }
 
@@ -1033,6 +1034,7 @@ int issue_partition_step(es_dg_t* const* parts, int P, const std::vector<int>& l
       a.rkA = kRkA[s];
       a.rkB = kRkB[s];
       a.dt = dt;
+      a.share = P;
       e = esdg_launch_volume(h->g, h->L, h->P, h->mixed, 1, a, h->stream);
       if (e != cudaSuccess) return cuda_status(e);
     }

@@ -355,6 +355,7 @@ struct EsdgVolArgs {
   double rkA, rkB, dt;
   int* status;           // mode 1: set to 1 when an updated state value is not finite or a
                          // density is not positive (null: not checked)
+  long long share;       // launches of this kind that run side by side (slabs of one mesh)
 };
 // The mixed volume kernel with a moving background (per-tile kernel; its own
 // translation unit): mode 0 writes rhs, mode 1 applies the LSRK stage.
@@ -368,7 +369,6 @@ struct EsdgMember {
   EsdgVolArgs a;       // q_in == q_io: the member's state; dq, geometry, face fluxes, dt
   const double* fgeo;  // face geometry
   const double* bg;    // mixed background (rho_bg, b_bg, p_bg, for the faces) or null
-  void* pad;
   // (sizeof a multiple of 16 bytes: the pipelined kernels bulk-copy descriptors)
 };
 

@@ -345,10 +345,10 @@ cudaError_t launch_volume64(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL&
                             const EsdgVolArgs& a, cudaStream_t s) {
   using SH = typename F64<N>::SH;
   constexpr auto k = k_volume64<N, MODE, false>;
-  const int cap = pipe_grid_cap<k>(SH::THREADS, F64<N>::SMEM);
-  if (cap < 0) return cudaErrorInvalidConfiguration;
+  const GridCap cap = pipe_grid_cap<k>(SH::THREADS, F64<N>::SMEM);
+  if (cap.ctas < 0) return cudaErrorInvalidConfiguration;
   int ntiles, grid, t1, s1;
-  pipe_split(g.E, SH::EPB, cap, ntiles, grid, t1, s1);
+  pipe_split(g.E, SH::EPB, cap.ctas, cap.sms / (int)a.share, ntiles, grid, t1, s1);
   if (ntiles == 0) return cudaSuccess;
   k<<<grid, SH::THREADS, F64<N>::SMEM, s>>>(pipe_member(g, P, a), nullptr, nullptr, nullptr, ntiles,
                                             L, a.rkA, a.rkB, esdg_take_phantom(), t1, s1);

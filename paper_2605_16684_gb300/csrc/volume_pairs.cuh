@@ -730,4 +730,62 @@ __device__ __forceinline__ bool stage32(float (&r)[5], const float* rbg, const E
   return bad;
 }
 
+// Launch helpers: the resident CTAs per device are found once per kernel
+// (the cache is keyed on the kernel itself, a template argument)
+struct GridCap {
+  int ctas, sms;  // resident CTAs and SMs of the device; ctas < 0: a CUDA error
+};
+template <auto k>
+GridCap pipe_grid_cap(int threads, size_t smem) {
+  constexpr int MAXDEV = 64;
+  static GridCap cap[MAXDEV];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAXDEV) return GridCap{-1, 0};
+  if (cap[dev].ctas == 0) {
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return GridCap{-1, 0};
+    int per_sm = 0, nsm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || per_sm < 1)
+      return GridCap{-1, 0};
+    cap[dev] = GridCap{per_sm * nsm, nsm};
+  }
+  return cap[dev];
+}
+
+// Tiles of a single mesh of E elements on a persistent grid of at most cap
+// CTAs: full rounds of EPB-element tiles, then the remaining elements as tiles
+// of s1 = ceil(rest / cap) elements, so the last round is spread over the grid.  A
+// mesh with fewer tiles than its share of the SMs (sms) is cut into tiles of
+// ceil(E / sms) elements: one SM's time grows with its tile's elements, so smaller
+// tiles on more SMs are faster although their warps are emptier (FP64 4^3 N = 3,
+// one LSRK step: 16 tiles of four elements 213 us, 64 of one 182 us).  Once every SM
+// has a tile the emptier warps cost more than the spread gives (four slabs of 330
+// elements, N = 4: one-element tiles 9 % slower than two-element ones).
+inline void pipe_split(int E, int EPB, int cap, int sms, int& ntiles, int& grid, int& t1, int& s1) {
+  const int nfull = (E + EPB - 1) / EPB;
+  grid = nfull < cap ? nfull : cap;
+  if (grid <= 0) {
+    ntiles = grid = t1 = 0;
+    s1 = 1;
+    return;
+  }
+  if (nfull < sms) {
+    s1 = (E + sms - 1) / sms;
+    t1 = 0;
+    ntiles = grid = (E + s1 - 1) / s1;
+    return;
+  }
+  t1 = (nfull / grid) * grid;  // tiles of the full rounds
+  if (t1 * EPB >= E) {         // no partial round
+    t1 = nfull;
+    s1 = EPB;
+    ntiles = nfull;
+    return;
+  }
+  const int rest = E - t1 * EPB;
+  s1 = (rest + grid - 1) / grid;
+  ntiles = t1 + (rest + s1 - 1) / s1;
+}
+
 }  // namespace esdg_vol

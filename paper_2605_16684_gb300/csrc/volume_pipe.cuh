@@ -493,49 +493,6 @@ __global__ void __launch_bounds__(PipeShape<N>::THREADS, 1)
   }
 }
 
-// Launch helpers: the resident CTAs per device are found once per kernel
-// (the cache is keyed on the kernel itself, a template argument)
-template <auto k>
-int pipe_grid_cap(int threads, size_t smem) {
-  constexpr int MAXDEV = 64;
-  static int cap[MAXDEV];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAXDEV) return -1;
-  if (cap[dev] == 0) {
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return -1;
-    int per_sm = 0, nsm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem) != cudaSuccess ||
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || per_sm < 1)
-      return -1;
-    cap[dev] = per_sm * nsm;
-  }
-  return cap[dev];
-}
-
-// Tiles of a single mesh of E elements on a persistent grid of at most cap
-// CTAs: full rounds of EPB-element tiles, then the remaining elements as tiles
-// of s1 = ceil(rest / cap) elements, so the last round is spread over the grid.
-inline void pipe_split(int E, int EPB, int cap, int& ntiles, int& grid, int& t1, int& s1) {
-  const int nfull = (E + EPB - 1) / EPB;
-  grid = nfull < cap ? nfull : cap;
-  if (grid <= 0) {
-    ntiles = grid = t1 = 0;
-    s1 = 1;
-    return;
-  }
-  t1 = (nfull / grid) * grid;  // tiles of the full rounds
-  if (t1 * EPB >= E) {         // no partial round
-    t1 = nfull;
-    s1 = EPB;
-    ntiles = nfull;
-    return;
-  }
-  const int rest = E - t1 * EPB;
-  s1 = (rest + grid - 1) / grid;
-  ntiles = t1 + (rest + s1 - 1) / s1;
-}
-
 inline EsdgMember pipe_member(const EsdgGrid& g, const EsdgPhys& P, const EsdgVolArgs& a) {
   EsdgMember m;
   memset(&m, 0, sizeof(m));
@@ -551,10 +508,10 @@ cudaError_t launch_pipe32(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL& L
                           const EsdgVolArgs& a, cudaStream_t s) {
   using SH = PipeShape<N>;
   constexpr auto k = k_volume_pipe32<N, MODE, false>;
-  const int cap = pipe_grid_cap<k>(SH::THREADS, Pipe32<N, MODE>::SMEM);
-  if (cap < 0) return cudaErrorInvalidConfiguration;
+  const GridCap cap = pipe_grid_cap<k>(SH::THREADS, Pipe32<N, MODE>::SMEM);
+  if (cap.ctas < 0) return cudaErrorInvalidConfiguration;
   int ntiles, grid, t1, s1;
-  pipe_split(g.E, SH::EPB, cap, ntiles, grid, t1, s1);
+  pipe_split(g.E, SH::EPB, cap.ctas, cap.sms / (int)a.share, ntiles, grid, t1, s1);
   if (ntiles == 0) return cudaSuccess;
   k<<<grid, SH::THREADS, Pipe32<N, MODE>::SMEM, s>>>(pipe_member(g, P, a), nullptr, nullptr, nullptr,
                                                      ntiles, L, a.rkA, a.rkB, esdg_take_phantom(),

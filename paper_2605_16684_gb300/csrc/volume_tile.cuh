@@ -8,17 +8,18 @@
 
 namespace esdg_vol {
 
-// One tile: elements e0 .. e0 + EPB - 1 of one mesh, processed by a CTA of
+// One tile: elements e0 .. e0 + ne - 1 of one mesh (ne <= EPB), processed by a CTA of
 // SH::THREADS threads with SH::SMEM bytes of shared memory at smraw.
 template <int N, int MODE, int BG, int EPB_ = 0>
 __device__ __forceinline__ void volume_tile(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL& L,
-                                            const EsdgVolArgs& a, int e0, unsigned char* smraw) {
+                                            const EsdgVolArgs& a, int e0, int ne,
+                                            unsigned char* smraw) {
   using SH = Shape<N, true, BG, EPB_>;
   using R = typename SH::R;
   constexpr int Nq = SH::Nq, NP = SH::NP, NPEN = SH::NPEN, EPB = SH::EPB, NF = SH::NF;
   constexpr int T = SH::THREADS;
   R* sm = reinterpret_cast<R*>(smraw);
-  const int E = g.E;
+  const int E = min(g.E, e0 + ne);
   const R* vg = reinterpret_cast<const R*>(a.vgeo);
   const double gm1 = P.gamma - 1.0;
   const float gm1f = esdg_d2f(gm1);
@@ -177,9 +178,9 @@ __device__ __forceinline__ void volume_tile(const EsdgGrid& g, const EsdgPhys& P
 
 template <int N, int MODE, int BG>
 __global__ void __launch_bounds__(Shape<N, true, BG>::THREADS)
-    k_volume(EsdgGrid g, EsdgPhys P, EsdgLGL L, EsdgVolArgs a) {
+    k_volume(EsdgGrid g, EsdgPhys P, EsdgLGL L, EsdgVolArgs a, int ne) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  volume_tile<N, MODE, BG>(g, P, L, a, blockIdx.x * Shape<N, true, BG>::EPB, smraw);
+  volume_tile<N, MODE, BG>(g, P, L, a, blockIdx.x * ne, ne, smraw);
 }
 
 // Persistent batched volume kernel: CTAs stride over a device work table of
@@ -207,7 +208,7 @@ __global__ void __launch_bounds__(Shape<N, true, BG, EPB_>::THREADS)
       mb.a.rkB = rkB;
     }
     __syncthreads();
-    volume_tile<N, 1, BG, EPB_>(mb.g, mb.P, L, mb.a, tile.y, smraw);
+    volume_tile<N, 1, BG, EPB_>(mb.g, mb.P, L, mb.a, tile.y, Shape<N, true, BG, EPB_>::EPB, smraw);
     __syncthreads();
   }
 }
@@ -216,17 +217,15 @@ template <int N, int MODE, int BG>
 cudaError_t launch_one(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL& L,
                        const EsdgVolArgs& a, cudaStream_t s) {
   using SH = Shape<N, true, BG>;
-  static bool configured = false;  // one-time attribute set per instantiation
-  if (!configured) {
-    cudaError_t err = cudaFuncSetAttribute(k_volume<N, MODE, BG>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)SH::SMEM);
-    if (err != cudaSuccess) return err;
-    configured = true;
-  }
-  const unsigned blocks = (unsigned)((g.E + SH::EPB - 1) / SH::EPB);
-  if (blocks == 0) return cudaSuccess;
-  k_volume<N, MODE, BG><<<blocks, SH::THREADS, SH::SMEM, s>>>(g, P, L, a);
+  constexpr auto k = k_volume<N, MODE, BG>;
+  const GridCap cap = pipe_grid_cap<k>(SH::THREADS, SH::SMEM);
+  if (cap.ctas < 0) return cudaErrorInvalidConfiguration;
+  // a mesh with fewer tiles than SMs: smaller tiles on more SMs (pipe_split)
+  const int sms = cap.sms / (int)a.share;
+  const int ne = g.E <= (sms - 1) * SH::EPB ? (g.E + sms - 1) / sms : SH::EPB;
+  if (g.E == 0) return cudaSuccess;
+  const unsigned blocks = (unsigned)((g.E + ne - 1) / ne);
+  k<<<blocks, SH::THREADS, SH::SMEM, s>>>(g, P, L, a, ne);
   return cudaGetLastError();
 }
 

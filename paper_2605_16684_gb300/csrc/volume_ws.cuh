@@ -503,10 +503,10 @@ cudaError_t launch_ws32(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL& L,
                         const EsdgVolArgs& a, cudaStream_t s) {
   using W = Ws32<N, MODE>;
   constexpr auto k = k_volume_ws32<N, MODE>;
-  const int cap = pipe_grid_cap<k>(W::T, W::SMEM);
-  if (cap < 0) return cudaErrorInvalidConfiguration;
+  const GridCap cap = pipe_grid_cap<k>(W::T, W::SMEM);
+  if (cap.ctas < 0) return cudaErrorInvalidConfiguration;
   int ntiles, grid, t1, s1;
-  pipe_split(g.E, W::EPB, cap, ntiles, grid, t1, s1);
+  pipe_split(g.E, W::EPB, cap.ctas, cap.sms / (int)a.share, ntiles, grid, t1, s1);
   if (ntiles == 0) return cudaSuccess;
   k<<<grid, W::T, W::SMEM, s>>>(pipe_member(g, P, a), ntiles, L, a.rkA, a.rkB, esdg_take_phantom(),
                                 t1, s1);
