@@ -734,12 +734,13 @@ int es_dg_rhs(es_dg_t* h, const double* q, double* rhs, int on_device) {
 
 int es_dg_cfl_dt(es_dg_t* h, double C, double* dt) {
   if (!h || !dt || !(C > 0.0)) return ES_DG_EINVAL;
-  cudaError_t e = esdg_launch_cfl(h->g, h->L, h->P, h->q, h->x, h->J, h->Ja, h->scratch, h->result,
+  cudaError_t e = esdg_launch_cfl(h->g, h->P, h->q, h->x, h->J, h->Ja, h->scratch, h->result,
                                   h->stream);
-  double r = 0.0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&r, h->result, sizeof(double), cudaMemcpyDeviceToHost, h->stream);
+  double lambda = 0.0;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&lambda, h->result, sizeof(double), cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cuda_status(e);
+  const double r = std::fmin(1e300, 1.0 / lambda);
   if (!(r > 0.0) || r != r) return ES_DG_ENAN;
   *dt = C * (h->L.xi[1] - h->L.xi[0]) * r;
   return ES_DG_OK;
