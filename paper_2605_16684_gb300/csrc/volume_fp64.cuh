@@ -68,7 +68,7 @@ __device__ __forceinline__ void pencil_rolled(R (&acc)[N + 1][5], const LOAD& lo
 
 template <int N, int MODE, bool TABLE>
 __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
-    k_volume64(const EsdgMember one, const EsdgMember* __restrict__ members,
+    k_volume64(const __grid_constant__ EsdgMember one, const EsdgMember* __restrict__ members,
                const int2* __restrict__ tiles, const int* __restrict__ ntiles_d, int ntiles_1,
                const __grid_constant__ EsdgLGL L, double rkA, double rkB, unsigned phantom, int t1,
                int s1) {
@@ -77,7 +77,6 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
   constexpr int Nq = SH::Nq, NP = SH::NP, NPEN = SH::NPEN, EPB = SH::EPB, NF = F64<N>::NF;
   constexpr int T = SH::THREADS;
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ __align__(16) EsdgMember M;
   __shared__ unsigned long long bar;
   __shared__ esdg_fx::FxElement fxe[EPB];
   // per element: its path; the pencils (three directions, 64
@@ -87,25 +86,16 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
   double* const xs = reinterpret_cast<double*>(smraw) + F64<N>::X0;
   const int tid = threadIdx.x;
   const int ntiles = TABLE ? *ntiles_d : ntiles_1;
-  int member = -1;
   if (tid == 0) {
     esdg_mbar_init(&bar, 1);
     esdg_fence_mbar_init();
-    if constexpr (!TABLE) M = one;
   }
   __syncthreads();
   unsigned parity = 0;
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, parity ^= 1u) {
-    if constexpr (TABLE) {
-      const int m = tiles[tile].x;
-      if (m != member) {
-        const int* src = reinterpret_cast<const int*>(members + m);
-        int* dst = reinterpret_cast<int*>(&M);
-        for (int k = tid; k < (int)(sizeof(EsdgMember) / sizeof(int)); k += T) dst[k] = src[k];
-        member = m;
-        __syncthreads();
-      }
-    }
+    // the descriptor stays in the constant bank (or global memory: a batch); in
+    // shared memory every store there would force its fields to be read again
+    const EsdgMember& M = TABLE ? members[tiles[tile].x] : one;
     const EsdgGrid& g = M.g;
     const EsdgPhys& P = M.P;
     const EsdgVolArgs& a = M.a;
@@ -350,7 +340,11 @@ cudaError_t launch_volume64(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL&
   int ntiles, grid, t1, s1;
   pipe_split(g.E, SH::EPB, cap.ctas, cap.sms / (int)a.share, ntiles, grid, t1, s1);
   if (ntiles == 0) return cudaSuccess;
-  k<<<grid, SH::THREADS, F64<N>::SMEM, s>>>(pipe_member(g, P, a), nullptr, nullptr, nullptr, ntiles,
+  // one CTA per tile: the hardware hands tiles out as CTAs end, so tiles of unequal
+  // cost (path, clock) leave no SM waiting for the CTA with the costliest share, as a
+  // persistent loop over a fixed share did (32^3 N = 4: 1.124 -> 0.976 ms; 16^3 N = 7:
+  // 0.790 -> 0.763)
+  k<<<ntiles, SH::THREADS, F64<N>::SMEM, s>>>(pipe_member(g, P, a), nullptr, nullptr, nullptr, ntiles,
                                             L, a.rkA, a.rkB, esdg_take_phantom(), t1, s1);
   return cudaGetLastError();
 }
