@@ -763,9 +763,10 @@ int es_dg_sync(es_dg_t* h) {
   if (!h) return ES_DG_EINVAL;
   const int st = cuda_status(cudaStreamSynchronize(h->stream));
   if (st != ES_DG_OK) return st;
-  const int t64 = esdg_volume_f64_take_timeout(), t32 = esdg_volume_mixed_take_timeout();
-  if (t64 < 0 || t32 < 0) return ES_DG_ECUDA;
-  if (t64 || t32) return ES_DG_ETIMEOUT;
+  const int t64 = esdg_volume_f64_take_timeout(), t32 = esdg_volume_mixed_take_timeout(),
+            t32o = esdg_volume_mixed_other_take_timeout();
+  if (t64 < 0 || t32 < 0 || t32o < 0) return ES_DG_ECUDA;
+  if (t64 || t32 || t32o) return ES_DG_ETIMEOUT;
   const int bad = esdg_take_status(h);
   if (bad < 0) return ES_DG_ECUDA;
   return bad ? ES_DG_ENAN : ES_DG_OK;

@@ -357,10 +357,10 @@ struct EsdgVolArgs {
                          // density is not positive (null: not checked)
   long long share;       // launches of this kind that run side by side (slabs of one mesh)
 };
-// The mixed volume kernel with a moving background (per-tile kernel; its own
+// The mixed volume kernel without a background or with a moving one (its own
 // translation unit): mode 0 writes rhs, mode 1 applies the LSRK stage.
-cudaError_t esdg_launch_volume_mixed_moving(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys& P,
-                                            int mode, const EsdgVolArgs& a, cudaStream_t s);
+cudaError_t esdg_launch_volume_mixed_other(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys& P,
+                                           int mode, const EsdgVolArgs& a, cudaStream_t s);
 // One mesh of a batch: everything its kernels need, read by the persistent
 // batched kernels from a device array (one entry per resident solve).
 struct EsdgMember {
@@ -369,13 +369,12 @@ struct EsdgMember {
   EsdgVolArgs a;       // q_in == q_io: the member's state; dq, geometry, face fluxes, dt
   const double* fgeo;  // face geometry
   const double* bg;    // mixed background (rho_bg, b_bg, p_bg, for the faces) or null
-  // (sizeof a multiple of 16 bytes: the pipelined kernels bulk-copy descriptors)
 };
 
 // Batched persistent launches over device work tables (tiles: int2 (member,
 // first element) for the volume, (member, first face node) in blocks of 256
 // for the faces; ntiles in device memory so the tables can change under a
-// captured graph).  variant selects the tile shape (elements per CTA).
+// captured graph).  variant selects the kernel (one at present).
 cudaError_t esdg_launch_face_batch(int N, int mixed, int bg, const EsdgMember* members,
                                    const int2* tiles, const int* ntiles, int grid, cudaStream_t s);
 // what: 0 launch (returns 0 or -1), 1 elements per tile, 2 CTAs per SM
@@ -392,10 +391,11 @@ int esdg_volume_batch_variants_mixed(int N);
 // pipelined volume launch registers on its first barrier without copying them;
 // read and cleared by the launcher.
 unsigned esdg_take_phantom();
-// 1 if a bounded wait of the pipelined FP64 / mixed volume kernels ran out
+// 1 if a bounded wait of the FP64 / mixed volume kernels ran out
 // since the last call (the flag is cleared), 0 if not, -1 on a CUDA error
 int esdg_volume_f64_take_timeout();
 int esdg_volume_mixed_take_timeout();
+int esdg_volume_mixed_other_take_timeout();
 cudaError_t esdg_launch_volume_f64(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys& P, int mode,
                                    const EsdgVolArgs& a, cudaStream_t s);
 cudaError_t esdg_launch_volume_mixed(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys& P,

@@ -1,25 +1,20 @@
-// volume32m.cu -- the mixed-precision volume kernel relative to a moving
-// background (a flow carried by the background, e.g. the channel's balanced
-// jet): FP32 pairs formed as differences against the background's fluxes
-// (pair32bgm), per-tile kernel for every order.
-#include "volume_tile.cuh"
+// volume32m.cu -- the mixed-precision volume kernel without a background or
+// relative to a moving one (a flow carried by the background, e.g. the channel's
+// balanced jet: FP32 pairs formed as differences against the background's
+// fluxes, pair32bgm).
+#include "volume_impl.cuh"
+#include "volume_mixed.cuh"
 
-cudaError_t esdg_launch_volume_mixed_moving(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys& P,
-                                            int mode, const EsdgVolArgs& a, cudaStream_t s) {
+int esdg_volume_mixed_other_take_timeout() { return esdg_vol::take_timeout(); }
+
+cudaError_t esdg_launch_volume_mixed_other(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys& P,
+                                           int mode, const EsdgVolArgs& a, cudaStream_t s) {
   using namespace esdg_vol;
-#define ESDG_MV(NN)                                                                   \
-  case NN:                                                                            \
-    return mode ? launch_one<NN, 1, 2>(g, P, L, a, s) : launch_one<NN, 0, 2>(g, P, L, a, s);
-  switch (g.N) {
-    ESDG_MV(1)
-    ESDG_MV(2)
-    ESDG_MV(3)
-    ESDG_MV(4)
-    ESDG_MV(5)
-    ESDG_MV(6)
-    ESDG_MV(7)
-    default:
-      return cudaErrorInvalidValue;
-  }
-#undef ESDG_MV
+  return for_order(g.N, cudaErrorInvalidValue, [&](auto n) {
+    if (a.bgq)
+      return mode ? launch_volume32<n.value, 1, 2>(g, P, L, a, s)
+                  : launch_volume32<n.value, 0, 2>(g, P, L, a, s);
+    return mode ? launch_volume32<n.value, 1, 0>(g, P, L, a, s)
+                : launch_volume32<n.value, 0, 0>(g, P, L, a, s);
+  });
 }

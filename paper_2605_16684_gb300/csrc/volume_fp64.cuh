@@ -1,5 +1,5 @@
-// volume_fp64.cuh -- the FP64 volume kernel: persistent CTAs of a few elements,
-// pairs in fixed point (volume_fx.cuh) or, for elements outside its range, FP64.
+// volume_fp64.cuh -- the FP64 volume kernel: one CTA per tile of a few elements
+// (a batch: persistent CTAs over its work table), pairs in fixed point (volume_fx.cuh) or, for elements outside its range, FP64.
 //
 // A tile's phases use different pipes: the prologue and the epilogue the FP64
 // pipe and memory, the pair pass the integer pipes.  The tile is therefore
@@ -35,36 +35,6 @@ struct F64 {
   static constexpr size_t SMEM = sizeof(double) * (size_t)(X0 + 6 * P + 4);
   static_assert(SH::NF == 18, "FP64 node fields");
 };
-
-struct OneIssuer {  // thread 0 issues the copies
-  static constexpr int FIRST = 0, COUNT = 1;
-  static __device__ __forceinline__ unsigned mask() { return 1u; }
-};
-
-// All pairs of one pencil.  Node i is paired with the nodes after it; its sum
-// is then complete, leaves through done(i, sum) and the sums move down by one,
-// so that the code holds N pair bodies instead of N (N + 1)/2.
-template <int N, typename R, typename LOAD, typename PAIR, typename DONE>
-__device__ __forceinline__ void pencil_rolled(R (&acc)[N + 1][5], const LOAD& load,
-                                              const PAIR& pair, const DONE& done) {
-  constexpr int Nq = N + 1;
-#pragma unroll 1
-  for (int i = 0; i < Nq; i++) {
-    const auto A = load(i);
-#pragma unroll
-    for (int k = 1; k < Nq; k++) {
-      if (i + k < Nq) {
-        const auto B = load(i + k);
-        pair(A, B, i, i + k, acc[0], acc[k]);
-      }
-    }
-    done(i, acc[0]);
-#pragma unroll
-    for (int k = 0; k < N; k++)
-#pragma unroll
-      for (int v = 0; v < 5; v++) acc[k][v] = acc[k + 1][v];
-  }
-}
 
 template <int N, int MODE, bool TABLE>
 __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
@@ -105,8 +75,7 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
     const int* const nscale = esdg_fx::metric_scales(vg, g.E, NP);
     if (tid == 0) {
       const double* q = a.q_in + (size_t)e0 * 5 * NP;
-      const BlockCopy bl[1] = {{xs, q, a.q_in + (size_t)g.E * 5 * NP, ne * 5 * NP, 8}};
-      pipe_issue<OneIssuer>(0, bl, 1, &bar, 0, nullptr, nullptr, phantom);
+      pipe_issue(BlockCopy{xs, q, a.q_in + (size_t)g.E * 5 * NP, ne * 5 * NP}, &bar, phantom);
       phantom = 0;
     }
     if (tid < EPB) {
@@ -124,7 +93,7 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
       esdg_cp_async(S + 18 * NP, gr + 10 * NP);
     }
     esdg_cp_async_wait_all();  // these, and thread 0's edge elements of q
-    const bool ok = esdg_mbar_wait(&bar, parity, ESDG_WAIT_LIMIT);
+    const bool ok = tile_wait(&bar, parity);
     if (__syncthreads_or(!ok)) {
       if (tid == 0) atomicExch(&g_esdg_vol_timeout, 1);
       return;
@@ -337,8 +306,8 @@ cudaError_t launch_volume64(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL&
   constexpr auto k = k_volume64<N, MODE, false>;
   const GridCap cap = pipe_grid_cap<k>(SH::THREADS, F64<N>::SMEM);
   if (cap.ctas < 0) return cudaErrorInvalidConfiguration;
-  int ntiles, grid, t1, s1;
-  pipe_split(g.E, SH::EPB, cap.ctas, cap.sms / (int)a.share, ntiles, grid, t1, s1);
+  int ntiles, t1, s1;
+  pipe_split(g.E, SH::EPB, cap.ctas, cap.sms / (int)a.share, ntiles, t1, s1);
   if (ntiles == 0) return cudaSuccess;
   // one CTA per tile: the hardware hands tiles out as CTAs end, so tiles of unequal
   // cost (path, clock) leave no SM waiting for the CTA with the costliest share, as a

@@ -1,8 +1,7 @@
 // volume_impl.cuh -- flux-differencing volume kernel (Section 3, the volume term
 // of Eq. (nm:semi), with the optimisations of Section 4.1).
-// The arithmetic lives in volume_pairs.cuh, the per-tile kernels in
-// volume_tile.cuh, the pipelined persistent kernels in volume_pipe.cuh; this
-// file dispatches the single-mesh launches.
+// The arithmetic lives in volume_pairs.cuh and volume_fx.cuh, the kernels in
+// volume_fp64.cuh and volume_mixed.cuh; this file dispatches on the order.
 //
 //   rhs_i = -(1/J_i) [ sum_d sum_l Dt^{(d)}_{il} H^d(q_i, q_l) + face lifts ] + h_i
 //
@@ -27,55 +26,32 @@
 // imbalance, no shuffles or atomics); the pencil's accumulators live in
 // registers and are exchanged once through shared memory.
 //
-// FP64: log means use the artanh series when u = f^2 < 1e-4 and per-node
-// logarithms otherwise (computed only for CTAs that need them).  Mixed: the
+// FP64: pairs in 60-bit fixed point where the element's fields fit it, else FP64
+// with the artanh series for log means when u = f^2 < 1e-4 and per-node logarithms
+// otherwise.  Mixed: the
 // prologue recovers the pressure in FP64 and stages FP32 node data; pairs,
 // sums and face lifts run in FP32; the log branch uses log1pf of the ratio;
 // the geopotential is carried relative to each element's first node.
 #pragma once
-#include "volume_fp64.cuh"
-#include "volume_pipe.cuh"
-#include "volume_tile.cuh"
-#include "volume_ws.cuh"
+#include <type_traits>
+
+#include "esdg_internal.cuh"
 
 namespace esdg_vol {
 
-template <bool MIXED>
-cudaError_t launch_volume_t(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys& P, int mode,
-                            const EsdgVolArgs& a, cudaStream_t s) {
-#define ESDG_CASE(NN)                                                          \
-  case NN:                                                                     \
-    if constexpr (!MIXED) {                                                    \
-      return mode ? launch_volume64<NN, 1>(g, P, L, a, s)                        \
-                  : launch_volume64<NN, 0>(g, P, L, a, s);                       \
-    }                                                                          \
-    if constexpr (MIXED) {                                                     \
-      if (a.bg && a.bgq) return esdg_launch_volume_mixed_moving(g, L, P, mode, a, s); \
-      if (a.bg) {                                                              \
-        if constexpr (WsCfg<NN>::ON && Ws32<NN, 1>::SMEM <= ESDG_PIPE_SMEM_MAX) \
-          return mode ? launch_ws32<NN, 1>(g, P, L, a, s)                      \
-                      : launch_ws32<NN, 0>(g, P, L, a, s);                     \
-        if constexpr (Pipe32<NN, 1>::SMEM <= ESDG_PIPE_SMEM_MAX)               \
-          return mode ? launch_pipe32<NN, 1>(g, P, L, a, s)                    \
-                      : launch_pipe32<NN, 0>(g, P, L, a, s);                   \
-        return mode ? launch_one<NN, 1, true>(g, P, L, a, s)            \
-                    : launch_one<NN, 0, true>(g, P, L, a, s);           \
-      }                                                                        \
-      return mode ? launch_one<NN, 1, false>(g, P, L, a, s)             \
-                  : launch_one<NN, 0, false>(g, P, L, a, s);            \
-    }
-  switch (g.N) {
-    ESDG_CASE(1)
-    ESDG_CASE(2)
-    ESDG_CASE(3)
-    ESDG_CASE(4)
-    ESDG_CASE(5)
-    ESDG_CASE(6)
-    ESDG_CASE(7)
-    default:
-      return cudaErrorInvalidValue;
+// f(std::integral_constant<int, N>) for the order N = 1..7, or `other`
+template <typename T, typename F>
+T for_order(int N, T other, const F& f) {
+  switch (N) {
+    case 1: return f(std::integral_constant<int, 1>{});
+    case 2: return f(std::integral_constant<int, 2>{});
+    case 3: return f(std::integral_constant<int, 3>{});
+    case 4: return f(std::integral_constant<int, 4>{});
+    case 5: return f(std::integral_constant<int, 5>{});
+    case 6: return f(std::integral_constant<int, 6>{});
+    case 7: return f(std::integral_constant<int, 7>{});
+    default: return other;
   }
-#undef ESDG_CASE
 }
 
 }  // namespace esdg_vol

@@ -2,8 +2,8 @@
 // (Section 3, Eq. (nm:semi); Section 4.1): tile shapes, node data, the two-point
 // pair in FP64 and FP32 (with and without a hydrostatic background), the pencil
 // pass, the interface lifts, the node prologues and the mixed stage update.
-// Shared by the per-tile kernels (volume_tile.cuh) and the pipelined
-// persistent kernels (volume_pipe.cuh), so both give bitwise the same results.
+// Used by the FP64 kernel (volume_fp64.cuh) and the mixed one (volume_mixed.cuh),
+// single meshes and batches alike, so both give bitwise the same results.
 #pragma once
 #include <cstring>
 #include <type_traits>
@@ -13,24 +13,12 @@
 
 namespace esdg_vol {
 
-
-// elements per CTA of the mixed kernels, chosen so that 3 Nq^2 EPB pencils fill
-// whole warps
-template <int N> struct Cfg;
-template <> struct Cfg<1> { static constexpr int EPB = 16; };
-template <> struct Cfg<2> { static constexpr int EPB = 16; };
-template <> struct Cfg<3> { static constexpr int EPB = 8; };
-template <> struct Cfg<4> { static constexpr int EPB = 5; };
-template <> struct Cfg<5> { static constexpr int EPB = 3; };
-template <> struct Cfg<6> { static constexpr int EPB = 2; };
-template <> struct Cfg<7> { static constexpr int EPB = 2; };
-
 // BG: 0 no background, 1 a background at rest (hydrostatic), 2 a moving
 // background (one that carries a flow; mixed mode only)
-template <int N, bool MIXED, int BG = 0, int EPB_ = 0>
+template <int N, bool MIXED, int BG, int EPB_>
 struct Shape {
   static constexpr int Nq = N + 1, NP = Nq * Nq * Nq, NPEN = Nq * Nq;
-  static constexpr int EPB = EPB_ > 0 ? EPB_ : Cfg<N>::EPB;  // elements per CTA (tile)
+  static constexpr int EPB = EPB_;  // elements per CTA (tile)
   static constexpr int PENCILS = 3 * NPEN * EPB;
   static constexpr int THREADS = ((PENCILS + 31) / 32) * 32;
   // node fields: rq=rho/4, bh=b/2, ib=1/b, uh=u/2 (3), ph=phi/2, [lr, lb], nh=Ja/2 (9),
@@ -443,25 +431,45 @@ __device__ __forceinline__ void pair32bgm(const Node<float>& A, const Node<float
   al[4] = fmaf(dli, FE, al[4]);
 }
 
-// every pair of one pencil in FP32; ce = 1/(2(gamma - 1))
-template <int N, bool LOGS, int BG>
-__device__ __forceinline__ void pencil_pass(const float* __restrict__ S, int d, int base, int stride,
-                                            const EsdgLGL& L, float ce, float (&acc)[N + 1][5]) {
-  using SH = Shape<N, true, BG>;
+// All pairs of one pencil.  Node i is paired with the nodes after it; its sum
+// is then complete, leaves through done(i, sum) and the sums move down by one,
+// so that the code holds N pair bodies instead of N (N + 1)/2.
+template <int N, typename R, typename LOAD, typename PAIR, typename DONE>
+__device__ __forceinline__ void pencil_rolled(R (&acc)[N + 1][5], const LOAD& load,
+                                              const PAIR& pair, const DONE& done) {
   constexpr int Nq = N + 1;
-#pragma unroll
+#pragma unroll 1
   for (int i = 0; i < Nq; i++) {
-    const Node<float> A = load_node<float, LOGS, SH::F_NH, SH::NP, BG>(S, base + i * stride, d);
+    const auto A = load(i);
 #pragma unroll
-    for (int l = i + 1; l < Nq; l++) {
-      const Node<float> B = load_node<float, LOGS, SH::F_NH, SH::NP, BG>(S, base + l * stride, d);
-      if constexpr (BG == 2)
-        pair32bgm<LOGS>(A, B, L.Dtf[i][l], L.Dtf[l][i], ce, acc[i], acc[l]);
-      else if constexpr (BG)
-        pair32bg<LOGS>(A, B, L.Dtf[i][l], L.Dtf[l][i], ce, acc[i], acc[l]);
-      else
-        pair32<LOGS>(A, B, L.Dtf[i][l], L.Dtf[l][i], ce, acc[i], acc[l]);
+    for (int k = 1; k < Nq; k++) {
+      if (i + k < Nq) {
+        const auto B = load(i + k);
+        pair(A, B, i, i + k, acc[0], acc[k]);
+      }
     }
+    done(i, acc[0]);
+#pragma unroll
+    for (int k = 0; k < N; k++)
+#pragma unroll
+      for (int v = 0; v < 5; v++) acc[k][v] = acc[k + 1][v];
+  }
+}
+
+// The same unrolled over i as well: no register moves and independent pairs side
+// by side, which the short FP32 pair needs (32^3 N = 4 mixed: 0.39 ms rolled).
+template <int N, typename R, typename LOAD, typename PAIR, typename DONE>
+__device__ __forceinline__ void pencil_unrolled(R (&acc)[N + 1][5], const LOAD& load,
+                                                const PAIR& pair, const DONE& done) {
+#pragma unroll
+  for (int i = 0; i <= N; i++) {
+    const auto A = load(i);
+#pragma unroll
+    for (int l = i + 1; l <= N; l++) {
+      const auto B = load(l);
+      pair(A, B, i, l, acc[i], acc[l]);
+    }
+    done(i, acc[i]);
   }
 }
 
@@ -512,17 +520,6 @@ __device__ double far_terms(const EsdgGrid& g, const EsdgVolArgs& a, int e, int 
     else sum += t.p[v];
   }
   return sum;
-}
-// Mixed path: the terms are added after the pair sums (once the element's
-// reference geopotential is restored in them); fetched before the pair pass,
-// their gathers' latency hides behind it.
-template <int N, typename R>
-__device__ __forceinline__ void face_add(const FaceTerms<R>& t, R (&acc)[N + 1][5]) {
-#pragma unroll
-  for (int v = 0; v < 5; v++) {
-    acc[0][v] -= t.m[v];
-    acc[N][v] += t.p[v];
-  }
 }
 // FP64 node primitives from the conserved state: rho/4, 1/b = 2p/rho, u/2,
 // phi/2 and p/2 (in the slot of ln b), with p = (gamma - 1)(E - rho phi -
@@ -686,33 +683,33 @@ __device__ __forceinline__ Prim32m prims32bgm(double q0, double q1, double q2, d
 // Mixed-precision stage update of one node: r = -(1/J) (volume + lifts) in
 // FP32, plus the background's right-hand side (stored in FP32) and the
 // Coriolis source, all in FP32 (they join an FP32 increment); FP64 only in
-// q += B dq.  Arrays are per node with stride NP between variables: rbg (3,
+// q += B dq.  Arrays are per node with stride SI between variables: rbg (3,
 // background momentum rhs; 5, the full rhs of a moving background), qin (5),
-// dqold (5) may be in shared or global memory; dq and qio are the node's
+// dqold (5) may be registers, shared or global memory; dq and qio are the node's
 // global locations; qbg (5) the moving background's state (its Coriolis force
 // is part of its rhs, so the source here acts on m - m_bg).  Returns true if
 // the updated state is not finite or its density is not positive.
-template <int NP, int BG>
+template <int NP, int BG, int SI = NP>
 __device__ __forceinline__ bool stage32(float (&r)[5], const float* rbg, const EsdgPhys& P,
                                         double y, const double* qin, const float* dqold, float* dq,
                                         double* qio, double rkA, double rkB, double dt,
                                         const double* qbg = nullptr) {
   if constexpr (BG == 2) {
 #pragma unroll
-    for (int v = 0; v < 5; v++) r[v] += rbg[v * NP];
+    for (int v = 0; v < 5; v++) r[v] += rbg[v * SI];
   } else if constexpr (BG) {
     r[1] += rbg[0];
-    r[2] += rbg[NP];
-    r[3] += rbg[2 * NP];
+    r[2] += rbg[SI];
+    r[3] += rbg[2 * SI];
   }
   if ((P.f0 != 0.0) || (P.beta != 0.0)) {
     const float f = esdg_d2f(P.f0 + P.beta * (y - P.y0));
     if constexpr (BG == 2) {
-      r[1] = fmaf(f, esdg_d2f(qin[2 * NP] - qbg[2 * NP]), r[1]);
-      r[2] = fmaf(-f, esdg_d2f(qin[NP] - qbg[NP]), r[2]);
+      r[1] = fmaf(f, esdg_d2f(qin[2 * SI] - qbg[2 * SI]), r[1]);
+      r[2] = fmaf(-f, esdg_d2f(qin[SI] - qbg[SI]), r[2]);
     } else {
-      r[1] = fmaf(f, esdg_d2f(qin[2 * NP]), r[1]);
-      r[2] = fmaf(-f, esdg_d2f(qin[NP]), r[2]);
+      r[1] = fmaf(f, esdg_d2f(qin[2 * SI]), r[1]);
+      r[2] = fmaf(-f, esdg_d2f(qin[SI]), r[2]);
     }
   }
   const float A = esdg_d2f(rkA), B = esdg_d2f(rkB), dtf = esdg_d2f(dt);
@@ -721,9 +718,9 @@ __device__ __forceinline__ bool stage32(float (&r)[5], const float* rbg, const E
   for (int v = 0; v < 5; v++) {
     // the first stage (A = 0) does not read the register: a register left
     // non-finite by an earlier diverged run must not poison a new one
-    const float dv = A == 0.0f ? dtf * r[v] : fmaf(A, dqold[(size_t)v * NP], dtf * r[v]);
+    const float dv = A == 0.0f ? dtf * r[v] : fmaf(A, dqold[(size_t)v * SI], dtf * r[v]);
     dq[(size_t)v * NP] = dv;
-    const double qn = qin[(size_t)v * NP] + esdg_f2d(B * dv);
+    const double qn = qin[(size_t)v * SI] + esdg_f2d(B * dv);
     qio[(size_t)v * NP] = qn;
     bad |= esdg_bad_state(qn, v == 0);
   }
@@ -753,27 +750,27 @@ GridCap pipe_grid_cap(int threads, size_t smem) {
   return cap[dev];
 }
 
-// Tiles of a single mesh of E elements on a persistent grid of at most cap
-// CTAs: full rounds of EPB-element tiles, then the remaining elements as tiles
-// of s1 = ceil(rest / cap) elements, so the last round is spread over the grid.  A
+// Tiles of a single mesh of E elements on a device that holds cap CTAs: full rounds
+// of EPB-element tiles, then the remaining elements as tiles of s1 = ceil(rest / cap)
+// elements, so the last round is spread over all SMs.  A
 // mesh with fewer tiles than its share of the SMs (sms) is cut into tiles of
 // ceil(E / sms) elements: one SM's time grows with its tile's elements, so smaller
 // tiles on more SMs are faster although their warps are emptier (FP64 4^3 N = 3,
 // one LSRK step: 16 tiles of four elements 213 us, 64 of one 182 us).  Once every SM
 // has a tile the emptier warps cost more than the spread gives (four slabs of 330
 // elements, N = 4: one-element tiles 9 % slower than two-element ones).
-inline void pipe_split(int E, int EPB, int cap, int sms, int& ntiles, int& grid, int& t1, int& s1) {
+inline void pipe_split(int E, int EPB, int cap, int sms, int& ntiles, int& t1, int& s1) {
   const int nfull = (E + EPB - 1) / EPB;
-  grid = nfull < cap ? nfull : cap;
+  const int grid = nfull < cap ? nfull : cap;
   if (grid <= 0) {
-    ntiles = grid = t1 = 0;
+    ntiles = t1 = 0;
     s1 = 1;
     return;
   }
   if (nfull < sms) {
     s1 = (E + sms - 1) / sms;
     t1 = 0;
-    ntiles = grid = (E + s1 - 1) / s1;
+    ntiles = (E + s1 - 1) / s1;
     return;
   }
   t1 = (nfull / grid) * grid;  // tiles of the full rounds
