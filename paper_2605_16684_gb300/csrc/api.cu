@@ -196,6 +196,7 @@ EsdgVolArgs vol_args(es_dg_t* h, const double* q_in, double* rhs_out) {
   a.dt = 0.0;
   a.status = h->status;
   a.share = 1;
+  a.after = 0;
   return a;
 }
 
@@ -226,13 +227,13 @@ int resolve_background(es_dg_t* h);
 // x faces come first, plane by plane (plane 0 is a partition's low cut, the last
 // x plane its high cut), then the y and z faces.
 enum { FACES_ALL = 0, FACES_INTERIOR = 1, FACES_CUT = 2 };
-int launch_faces(es_dg_t* h, const double* q_in, int which) {
+int launch_faces(es_dg_t* h, const double* q_in, int which, int after = 0) {
   const bool moving = h->mixed && h->has_bg && h->bg_moving;
   const double* bg = (h->mixed && h->has_bg) ? h->bg : nullptr;
   const EsdgTraces tr = traces_of(h);
   auto run = [&](long long f0, long long f1) {
     return esdg_launch_face(h->g, h->P, h->mixed, q_in, h->fgeo, h->fflux, h->stream, bg, tr,
-                            moving ? h->bgq : nullptr, f0, f1);
+                            moving ? h->bgq : nullptr, f0, f1, after);
   };
   const long long plane = (long long)h->g.K[1] * h->g.K[2];
   const long long x0 = h->g.face_off[0], x1 = h->g.face_off[1];
@@ -250,20 +251,22 @@ int launch_faces(es_dg_t* h, const double* q_in, int which) {
   return cuda_status(e);
 }
 
-// face fluxes then volume (+ lift, source, optional RK update) for state q_in
+// face fluxes then volume (+ lift, source, optional RK update) for state q_in; after:
+// the launch before these in the stream is a stage's volume kernel
 int launch_stage(es_dg_t* h, const double* q_in, int mode, double* rhs_out, double A, double B,
-                 double dt) {
+                 double dt, int after = 0) {
   if (!traces_ready(h)) return ES_DG_EINVAL;
   if (h->bg_pending) {
     const int st = resolve_background(h);
     if (st) return st;
   }
-  const int stf = launch_faces(h, q_in, FACES_ALL);
+  const int stf = launch_faces(h, q_in, FACES_ALL, after);
   if (stf) return stf;
   EsdgVolArgs a = vol_args(h, q_in, rhs_out);
   a.rkA = A;
   a.rkB = B;
   a.dt = dt;
+  a.after = 1;
   const cudaError_t e = esdg_launch_volume(h->g, h->L, h->P, h->mixed, mode, a, h->stream);
   return cuda_status(e);
 }
@@ -751,7 +754,7 @@ int es_dg_step(es_dg_t* h, double dt, int nsteps) {
   if (is_partition(h)) return ES_DG_EINVAL;  // stages need the trace exchange
   for (int n = 0; n < nsteps; n++)
     for (int s = 0; s < 5; s++) {
-      int st = launch_stage(h, h->q, 1, nullptr, kRkA[s], kRkB[s], dt);
+      int st = launch_stage(h, h->q, 1, nullptr, kRkA[s], kRkB[s], dt, n + s > 0);
       if (st) return st;
     }
   return ES_DG_OK;

@@ -654,6 +654,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == sizeof(float) ? 4 : 1)
   // face nodes t0 .. t1 - 1 (global face-node indices); a launch over every
   // face takes them in the layered order
   constexpr long long NF2 = (N + 1) * (N + 1);
+  esdg_wait_before();
   long long tid = t0 + (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (tid >= t1) return;
   if (t0 == 0 && t1 == g.nfaces * NF2) {
@@ -723,24 +724,29 @@ __global__ void __launch_bounds__(256) k_face_batch(const EsdgMember* __restrict
 template <typename R, int BG>
 cudaError_t launch_face_t(const EsdgGrid& g, const EsdgPhys& P, const double* q, const double* fgeo,
                           R* fflux, const double* bg, EsdgTraces tr, cudaStream_t s,
-                          const double* bgq, long long f0, long long f1) {
+                          const double* bgq, long long f0, long long f1, int after) {
   const long long nf2 = (long long)g.Nq * g.Nq;
   if (f1 < 0 || f1 > g.nfaces) f1 = g.nfaces;
   if (f0 < 0) f0 = 0;
   if (f1 <= f0) return cudaSuccess;
   const long long t0 = f0 * nf2, t1 = f1 * nf2;
-  const unsigned blocks = (unsigned)((t1 - t0 + 255) / 256);
+  constexpr unsigned T = 256;
+  const unsigned blocks = (unsigned)((t1 - t0 + T - 1) / T);
+#define ESDG_F(NN)                                                                               \
+  case NN:                                                                                       \
+    return esdg_launch(k_face<R, NN, BG>, after, blocks, T, 0, s, g, P, q, fgeo, fflux, bg, tr, \
+                       bgq, t0, t1);
   switch (g.N) {
-    case 1: k_face<R, 1, BG><<<blocks, 256, 0, s>>>(g, P, q, fgeo, fflux, bg, tr, bgq, t0, t1); break;
-    case 2: k_face<R, 2, BG><<<blocks, 256, 0, s>>>(g, P, q, fgeo, fflux, bg, tr, bgq, t0, t1); break;
-    case 3: k_face<R, 3, BG><<<blocks, 256, 0, s>>>(g, P, q, fgeo, fflux, bg, tr, bgq, t0, t1); break;
-    case 4: k_face<R, 4, BG><<<blocks, 256, 0, s>>>(g, P, q, fgeo, fflux, bg, tr, bgq, t0, t1); break;
-    case 5: k_face<R, 5, BG><<<blocks, 256, 0, s>>>(g, P, q, fgeo, fflux, bg, tr, bgq, t0, t1); break;
-    case 6: k_face<R, 6, BG><<<blocks, 256, 0, s>>>(g, P, q, fgeo, fflux, bg, tr, bgq, t0, t1); break;
-    case 7: k_face<R, 7, BG><<<blocks, 256, 0, s>>>(g, P, q, fgeo, fflux, bg, tr, bgq, t0, t1); break;
+    ESDG_F(1)
+    ESDG_F(2)
+    ESDG_F(3)
+    ESDG_F(4)
+    ESDG_F(5)
+    ESDG_F(6)
+    ESDG_F(7)
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
+#undef ESDG_F
 }
 
 }  // namespace
@@ -763,14 +769,15 @@ cudaError_t esdg_launch_face_batch(int N, int mixed, int bg, const EsdgMember* m
 
 cudaError_t esdg_launch_face(const EsdgGrid& g, const EsdgPhys& P, int mixed, const double* q,
                              const double* fgeo, void* fflux, cudaStream_t s, const double* bg,
-                             EsdgTraces tr, const double* bgq, long long f0, long long f1) {
+                             EsdgTraces tr, const double* bgq, long long f0, long long f1,
+                             int after) {
   if (mixed && bg && bgq)
-    return launch_face_t<float, 2>(g, P, q, fgeo, (float*)fflux, bg, tr, s, bgq, f0, f1);
+    return launch_face_t<float, 2>(g, P, q, fgeo, (float*)fflux, bg, tr, s, bgq, f0, f1, after);
   if (mixed && bg)
-    return launch_face_t<float, 1>(g, P, q, fgeo, (float*)fflux, bg, tr, s, nullptr, f0, f1);
+    return launch_face_t<float, 1>(g, P, q, fgeo, (float*)fflux, bg, tr, s, nullptr, f0, f1, after);
   if (mixed)
-    return launch_face_t<float, 0>(g, P, q, fgeo, (float*)fflux, nullptr, tr, s, nullptr, f0, f1);
-  return launch_face_t<double, 0>(g, P, q, fgeo, (double*)fflux, nullptr, tr, s, nullptr, f0, f1);
+    return launch_face_t<float, 0>(g, P, q, fgeo, (float*)fflux, nullptr, tr, s, nullptr, f0, f1, after);
+  return launch_face_t<double, 0>(g, P, q, fgeo, (double*)fflux, nullptr, tr, s, nullptr, f0, f1, after);
 }
 
 cudaError_t esdg_launch_trace_pack(const EsdgGrid& g, const double* q, const double* bg, int nv,

@@ -55,6 +55,7 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
   double* const sm = reinterpret_cast<double*>(smraw) + F64<N>::S0;
   double* const xs = reinterpret_cast<double*>(smraw) + F64<N>::X0;
   const int tid = threadIdx.x;
+  if constexpr (!TABLE) esdg_wait_before();
   const int ntiles = TABLE ? *ntiles_d : ntiles_1;
   if (tid == 0) {
     esdg_mbar_init(&bar, 1);
@@ -307,15 +308,14 @@ cudaError_t launch_volume64(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL&
   const GridCap cap = pipe_grid_cap<k>(SH::THREADS, F64<N>::SMEM);
   if (cap.ctas < 0) return cudaErrorInvalidConfiguration;
   int ntiles, t1, s1;
-  pipe_split(g.E, SH::EPB, cap.ctas, cap.sms / (int)a.share, ntiles, t1, s1);
+  pipe_split(g.E, SH::EPB, cap.ctas, cap.sms / a.share, ntiles, t1, s1);
   if (ntiles == 0) return cudaSuccess;
   // one CTA per tile: the hardware hands tiles out as CTAs end, so tiles of unequal
   // cost (path, clock) leave no SM waiting for the CTA with the costliest share, as a
   // persistent loop over a fixed share did (32^3 N = 4: 1.124 -> 0.976 ms; 16^3 N = 7:
   // 0.790 -> 0.763)
-  k<<<ntiles, SH::THREADS, F64<N>::SMEM, s>>>(pipe_member(g, P, a), nullptr, nullptr, nullptr, ntiles,
-                                            L, a.rkA, a.rkB, esdg_take_phantom(), t1, s1);
-  return cudaGetLastError();
+  return esdg_launch(k, a.after, ntiles, SH::THREADS, F64<N>::SMEM, s, pipe_member(g, P, a), nullptr,
+                     nullptr, nullptr, ntiles, L, a.rkA, a.rkB, esdg_take_phantom(), t1, s1);
 }
 
 // batched (TABLE) launches; what: 0 launch (0 / -1), 1 elements per tile, 2 CTAs per SM

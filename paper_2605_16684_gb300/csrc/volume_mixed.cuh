@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(Mix<N, BG>::SH::THREADS, MixCfg<N, BG>::MINB)
   float* const xs = sm + Mix<N, BG>::X0;
   float* const js = sm + Mix<N, BG>::J0;
   const int tid = threadIdx.x;
+  if constexpr (!TABLE) esdg_wait_before();
   if (tid == 0) {
     esdg_mbar_init(&bar, 1);
     esdg_fence_mbar_init();
@@ -342,13 +343,12 @@ cudaError_t launch_volume32(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL&
   const GridCap cap = pipe_grid_cap<k>(SH::THREADS, Mix<N, BG>::SMEM);
   if (cap.ctas < 0) return cudaErrorInvalidConfiguration;
   int ntiles, t1, s1;
-  pipe_split(g.E, SH::EPB, cap.ctas, cap.sms / (int)a.share, ntiles, t1, s1);
+  pipe_split(g.E, SH::EPB, cap.ctas, cap.sms / a.share, ntiles, t1, s1);
   if (ntiles == 0) return cudaSuccess;
   // one CTA per tile: the hardware hands tiles out as CTAs end, which beats a
   // persistent loop over a fixed share (32^3 N = 4: 0.363 against 0.391 ms)
-  k<<<ntiles, SH::THREADS, Mix<N, BG>::SMEM, s>>>(pipe_member(g, P, a), nullptr, nullptr, nullptr,
-                                                ntiles, L, a.rkA, a.rkB, esdg_take_phantom(), t1, s1);
-  return cudaGetLastError();
+  return esdg_launch(k, a.after, ntiles, SH::THREADS, Mix<N, BG>::SMEM, s, pipe_member(g, P, a),
+                     nullptr, nullptr, nullptr, ntiles, L, a.rkA, a.rkB, esdg_take_phantom(), t1, s1);
 }
 
 // batched (TABLE) launches (members with a background at rest); what: 0 launch
