@@ -642,9 +642,16 @@ __device__ __forceinline__ long long face_layered(const EsdgGrid& g, long long w
   return g.face_off[2] + ((long long)k * K1 + b) * K0 + (r - b * K0);
 }
 
-// mixed: at most 64 registers, four 256-thread CTAs per SM
+// FP64: bounded by the FP64 pipe (about 180 operations a face node, 64 cycles a warp
+// instruction on an SM's quarter); mixed: by issue, at most 64 registers.  Nothing is
+// shared between the nodes of a CTA, so CTAs are two warps: a small mesh's face nodes
+// then spread over every SM, and a large one's last wave is short.  CTAs of 256 -> 64
+// threads, one LSRK step: FP64 4^3 N = 3 (3840 face nodes, 15 CTAs -> 60) 155 -> 124 us;
+// one right-hand side 13x9x7 N = 5 119 -> 113 us; mixed 32^3 N = 4 2106 -> 2085 us, FP64
+// 8787 -> 8772 us.  128 threads lie between, 32 within 1 % of 64.
+constexpr int FACE_THREADS = 64;
 template <typename R, int N, int BG>
-__global__ void __launch_bounds__(256, sizeof(R) == sizeof(float) ? 4 : 1)
+__global__ void __launch_bounds__(FACE_THREADS, sizeof(R) == sizeof(float) ? 1024 / FACE_THREADS : 1)
     k_face(EsdgGrid g, EsdgPhys P, const double* __restrict__ q,
                                               const double* __restrict__ fgeo,
                                               R* __restrict__ fflux,
@@ -730,7 +737,7 @@ cudaError_t launch_face_t(const EsdgGrid& g, const EsdgPhys& P, const double* q,
   if (f0 < 0) f0 = 0;
   if (f1 <= f0) return cudaSuccess;
   const long long t0 = f0 * nf2, t1 = f1 * nf2;
-  constexpr unsigned T = 256;
+  constexpr unsigned T = FACE_THREADS;
   const unsigned blocks = (unsigned)((t1 - t0 + T - 1) / T);
 #define ESDG_F(NN)                                                                               \
   case NN:                                                                                       \
