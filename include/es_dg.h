@@ -183,7 +183,7 @@ int es_dg_cfl_dt(es_dg_t* h, double C, double* dt);
 int es_dg_step(es_dg_t* h, double dt, int nsteps);
 
 /* Wait for the handle's stream.  Returns ES_DG_ETIMEOUT if, since the last
- * call, a bounded device wait of the pipelined volume kernels ran out (their
+ * call, a bounded device wait of the volume kernels ran out (their
  * tile copies never completed; the kernel stopped and the state is not
  * valid), ES_DG_ENAN if a stage update of this handle (es_dg_step) produced a
  * state value that is an infinity or a NaN, or a density that is not positive
