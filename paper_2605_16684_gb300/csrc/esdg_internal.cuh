@@ -422,7 +422,7 @@ int esdg_volume_batch_variants_f64(int N);
 int esdg_volume_batch_variants_mixed(int N);
 
 // Test hook (es_dg_debug_inject_wait_timeout): bytes the next single-mesh
-// pipelined volume launch registers on its first barrier without copying them;
+// volume launch registers on its first barrier without copying them;
 // read and cleared by the launcher.
 unsigned esdg_take_phantom();
 // 1 if a bounded wait of the FP64 / mixed volume kernels ran out

@@ -1,9 +1,10 @@
 // volume_fp64.cuh -- the FP64 volume kernel: one CTA per tile of a few elements
-// (a batch: persistent CTAs over its work table), pairs in fixed point (volume_fx.cuh) or, for elements outside its range, FP64.
+// (a batch: persistent CTAs over its work table), pairs in fixed point
+// (volume_fx.cuh) or, for elements outside its range, FP64.
 //
 // A tile's phases use different pipes: the prologue and the epilogue the FP64
 // pipe and memory, the pair pass the integer pipes.  The tile is therefore
-// small (about 192 threads) and several CTAs share an SM, so that one CTA's
+// small (64 to 224 threads) and several CTAs share an SM, so that one CTA's
 // prologue and epilogue run under another's pair pass.
 #pragma once
 #include "volume_pipe.cuh"
@@ -11,10 +12,14 @@
 namespace esdg_vol {
 
 // Elements per tile and the CTAs planned per SM (MINB; it sets the register
-// budget).  Measured at N = 4, 32^3: two elements and three CTAs (128 registers)
-// 1.21 ms, two CTAs (168 registers) 1.29 ms, one element and five CTAs (a third of
-// the third warp idle) 1.49 ms, four elements and one CTA 1.50 ms.  N = 5: two
-// elements (216 of 224 lanes) 0.513 ms against one (108 of 128) 0.526 ms at 20^3.
+// budget).  One launch, ms (EPB/MINB): N = 4, 32^3: 3/2 0.951, 2/3 0.972, 4/2 1.004, 2/4
+// 1.065, 2/2 1.154, 1/6 1.278; N = 5, 20^3: 2/2 0.455, 1/4 0.482; N = 6, 20^3: 1/2 1.010,
+// 2/1 1.189; N = 7, 16^3: 1/2 0.762, 1/3 0.928.  Up to N = 3 more and smaller CTAs are
+// faster on large meshes (N = 1, 64^3: 8/7 0.368 against 16/2 0.538; N = 2, 48^3: 2/10
+// 0.590 against 7/2 0.685; N = 3, 32^3: 2/6 0.498 against 4/2 0.530) but their fewer
+// registers lengthen a tile, which a mesh of one round of tiles waits for (N = 3, 6^3:
+// 0.0207 against 0.0162; N = 1, 13^3: 0.0123 against 0.0105; a 4^3 N = 3 step 126 against
+// 116 us), so the tiles with registers stay.
 template <int N> struct F64Cfg;
 template <> struct F64Cfg<1> { static constexpr int EPB = 16, MINB = 2; };
 template <> struct F64Cfg<2> { static constexpr int EPB = 7, MINB = 2; };

@@ -14,7 +14,7 @@
 // beyond.  Whole kernel, before (FP64 pairs) and after, one launch: 32^3 N = 4 warped bubble
 // 3.400 -> 1.164 ms (narrow path), 16^3 N = 7 2.77 -> 0.79 ms, 16^3 N = 4 on a 2 km
 // box 0.494 -> 0.209 ms (wide path), 60 x 12 x 6 N = 4 channel 0.566 -> 0.233 ms
-// (tall path).
+// (tall path); with the launches of volume_fp64.cuh 0.973, 0.762 and 0.189 ms.
 //
 // Which elements take it (fx_path, fx_scales), decided per element so that a
 // result does not depend on the tile: all densities and 1/b = 2p/rho positive and
