@@ -271,11 +271,9 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
         const double z0 = Z[0], z1 = Z[zs], z2 = Z[2 * zs];
         double r;
         if (!general) {
-          // the power of two on the exponent of the scale factor
           const int so = fxe[el2].out[v == 0 ? 0 : (v == 4 ? 2 : 1)];
-          const double ss = __hiloint2double(__double2hiint(sJ) - so * (1 << 20), __double2loint(sJ));
-          r = ss * (double)(__double_as_longlong(z0) + __double_as_longlong(z1) +
-                            __double_as_longlong(z2));
+          r = sJ * esdg_fx::from_fx(__double_as_longlong(z0) + __double_as_longlong(z1) +
+                                        __double_as_longlong(z2), so);
           if (any_far) r = fma(sJ, far_terms<N>(g, a, e2, n, v, far_lift[el2]), r);
         } else {
           r = sJ * (z0 + z1 + z2);

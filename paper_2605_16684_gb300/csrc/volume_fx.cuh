@@ -257,6 +257,14 @@ __device__ __forceinline__ i64 to_fx64(double v, int s) {
   return hi < 0 ? -(i64)m : (i64)m;
 }
 __device__ __forceinline__ Fx to_fx(double v, int s) { return limbs(to_fx64(v, s)); }
+// v 2^-s, |s| < 700 (a sum's scale lies between -250 and 620): the power of two goes
+// on the exponent field of the converted sum, which is zero or at least 1.  On the
+// factor that multiplies it (-dt/J) it would not do: a step of zero, a subnormal or an
+// infinite one has no exponent to add to.
+__device__ __forceinline__ double from_fx(i64 v, int s) {
+  const double d = (double)v;
+  return __hiloint2double(v ? __double2hiint(d) - s * (1 << 20) : 0, __double2loint(d));
+}
 // does v 2^s leave the limbs' range by 2^-b? (infinities and NaNs do)
 __device__ __forceinline__ bool fx_over(double v, int s, int b) {
   return ((__double2hiint(v) >> 20) & 0x7ff) > 1082 - s - b;
