@@ -3,7 +3,7 @@
 // Data layout in HBM (one handle, E elements, np = Nq^3 nodes each):
 //   q, dq, rhs      double [E][5][np]            element-major, variable, node
 //   vgeo            double [E][11][np]           1/2 Ja^d_c (9, fixed-point limbs), 1/J, phi;
-//                                                then int [E], the limbs' scales (volume_fx.cuh)
+//                                                then int [E][3], the limbs' scales (volume_fx.cuh)
 //   vgeo32          float  [E][11][np]           the same in FP32 (mixed mode)
 //   x               double [E][3][np]            node coordinates
 //   fgeo            double [F][5][Nq^2]          nhat (3), s / w_end, phi per face node
@@ -21,7 +21,7 @@
 #define ESDG_MAXNQ 8
 #define ESDG_NVGEO 11
 // bytes of vgeo
-#define ESDG_VGEO_BYTES(E, np) ((E) * ESDG_NVGEO * (np) * sizeof(double) + (E) * sizeof(int))
+#define ESDG_VGEO_BYTES(E, np) ((E) * ESDG_NVGEO * (np) * sizeof(double) + (E) * 3 * sizeof(int))
 
 struct EsdgLGL {  // LGL operators, passed by value (lives in the constant bank)
   int N;

@@ -123,23 +123,42 @@ __global__ void k_geometry(EsdgGrid g, EsdgLGL L, EsdgPhys P, double* __restrict
       }
     }
   }
-  // the FP64 path's metric terms in limbs of the element's common scale
-  __shared__ unsigned top;
+  // the FP64 path's metric terms in limbs, each component at the element's own scale
+  __shared__ unsigned top, col[3];
+  __shared__ int stretch[3];
+  if (threadIdx.x < 3) col[threadIdx.x] = 0u;
   if (threadIdx.x == 0) top = 0u;
   __syncthreads();
   double* vg = vgeo + (size_t)e * ESDG_NVGEO * np;
+  auto mag = [](double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; };
+  unsigned hc[3] = {0u, 0u, 0u};
+  for (int k = threadIdx.x; k < 3 * np; k += blockDim.x) {
+    const double* a = vg + (size_t)(k / np) * 3 * np + k % np;
+    for (int c = 0; c < 3; c++) hc[c] = max(hc[c], mag(a[c * np]));
+  }
+  for (int c = 0; c < 3; c++) atomicMax(&col[c], hc[c]);
+  __syncthreads();
+  if (threadIdx.x == 0) esdg_fx::metric_stretch(col, stretch);
+  __syncthreads();
   unsigned hi = 0u;
   for (int k = threadIdx.x; k < 3 * np; k += blockDim.x) {
     const double* a = vg + (size_t)(k / np) * 3 * np + k % np;
-    hi = max(hi, (unsigned)__double2hiint(a[0] * a[0] + a[np] * a[np] + a[2 * np] * a[2 * np]) & 0x7fffffffu);
+    double v = 0.0;
+    for (int c = 0; c < 3; c++) {
+      const double t = ldexp(a[c * np], -stretch[c]);
+      v += t * t;
+    }
+    hi = max(hi, mag(v));
   }
   atomicMax(&top, hi);
   __syncthreads();
-  const int sn = esdg_fx::metric_scale(top);
-  if (threadIdx.x == 0) esdg_fx::metric_scales(vgeo, g.E, np)[e] = sn;
-  if (sn == esdg_fx::FX_NO_METRIC) return;
+  const int sn = esdg_fx::metric_scale(top, stretch);
+  const bool none = sn == esdg_fx::FX_NO_METRIC;
+  if (threadIdx.x < 3)
+    esdg_fx::metric_scales(vgeo, g.E, np)[(size_t)e * 3 + threadIdx.x] = none ? sn : sn - stretch[threadIdx.x];
+  if (none) return;
   for (int k = threadIdx.x; k < 9 * np; k += blockDim.x)
-    esdg_fx::st_fx(vg + k, esdg_fx::to_fx(vg[k], sn));
+    esdg_fx::st_fx(vg + k, esdg_fx::to_fx(vg[k], sn - stretch[k / np % 3]));
 }
 
 // Face normals from the metric of the element on the face's "-" side (or the

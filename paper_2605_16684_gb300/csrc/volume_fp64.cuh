@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
       phantom = 0;
     }
     if (tid < EPB) {
+      if (tid < ne) esdg_fx::fx_metric(fxe[tid], nscale + 3 * (size_t)(e0 + tid));
       fxe[tid].mu = fxe[tid].mf = 0u;
       gen[tid] = 0u;
       for (int w = 0; w < 6; w++) far_lift[tid][w / 2][w % 2] = 0u;
@@ -108,15 +109,17 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
     {
       const double* qr0 = xs + esdg_block_shift(a.q_in + (size_t)e0 * 5 * NP);
       const double gm1 = P.gamma - 1.0;
-      auto mag = [](double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; };
       for (int idx = tid; idx < ne * NP; idx += T) {
         const int el = idx / NP, n = idx - el * NP;
         double* S = sm + (size_t)el * NF * NP;
         const double* qr = qr0 + (size_t)el * 5 * NP;
         prims64<NP>(qr[n], qr[NP + n], qr[2 * NP + n], qr[3 * NP + n], qr[4 * NP + n],
                     S[18 * NP + n], gm1, S, n);
-        atomicMax(&fxe[el].mu, max(mag(S[3 * NP + n]), max(mag(S[4 * NP + n]), mag(S[5 * NP + n]))));
-        atomicMax(&fxe[el].mf, mag(S[6 * NP + n]));
+        const int* k = fxe[el].sc.k;
+        using esdg_fx::stretched;
+        atomicMax(&fxe[el].mu, max(stretched(S[3 * NP + n], k[0]), max(stretched(S[4 * NP + n], k[1]),
+                                                                       stretched(S[5 * NP + n], k[2]))));
+        atomicMax(&fxe[el].mf, (unsigned)__double2hiint(S[6 * NP + n]) & 0x7fffffffu);
       }
     }
     __syncthreads();  // the copy of q consumed
@@ -127,7 +130,7 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
       const unsigned path = esdg_fx::fx_path(S[n], S[2 * NP + n], S[0], S[2 * NP]);
       if (path != esdg_fx::FX_NARROW) atomicMax(&gen[el], path);
       if (n == 0) {
-        esdg_fx::fx_scales(fxe[el], S[0], S[2 * NP], nscale[e0 + el], P.gamma - 1.0, P.igm1, L.wm);
+        esdg_fx::fx_scales(fxe[el], S[0], S[2 * NP], P.gamma - 1.0, P.igm1, L.wm);
         if (!fxe[el].sc.ok) atomicMax(&gen[el], (unsigned)esdg_fx::FX_GENERAL);
       }
     }
@@ -159,11 +162,11 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
       if (gen[el] != esdg_fx::FX_GENERAL) {
         using esdg_fx::i64;
         const esdg_fx::FxElement& E2 = fxe[el];
-        const int ks = E2.sc.s1;
+        const int ks[3] = {E2.sc.s1[0], E2.sc.s1[1], E2.sc.s1[2]};
         i64 acc[Nq][5];
 #pragma unroll
         for (int v = 0; v < 5; v++) {
-          const int so = E2.out[v == 0 ? 0 : (v == 4 ? 2 : 1)];
+          const int so = E2.out[v];
           far |= esdg_fx::fx_over(ft.m[v], so, 3) || esdg_fx::fx_over(ft.p[v], so, 3);
 #pragma unroll
           for (int i = 0; i < Nq; i++) acc[i][v] = 0;
@@ -188,19 +191,27 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
           om[NP + n] = out(2);
           om[2 * NP + n] = out(3);
         };
-        auto pass = [&](auto path) {
+        auto pass = [&](auto path, auto flat) {
           pencil_rolled<N>(acc, load,
                            [&](const esdg_fx::FxNode& A, const esdg_fx::FxNode& B, int i, int l,
                                i64* ai, i64* al) {
-                             esdg_fx::pair_fx<decltype(path)::value>(
+                             esdg_fx::pair_fx<decltype(path)::value, decltype(flat)::value>(
                                  A, B, esdg_fx::Fx{L.Qh[i][l], L.Ql[i][l]}, ks,
                                  esdg_fx::Round{L.rnd[0], L.rnd[1]}, ai, al);
                            }, done);
         };
-        using namespace esdg_fx;
-        if (gen[el] == FX_NARROW) pass(std::integral_constant<int, FX_NARROW>{});
-        else if (gen[el] == FX_WIDE) pass(std::integral_constant<int, FX_WIDE>{});
-        else pass(std::integral_constant<int, FX_TALL>{});
+        auto take = [&](auto flat) {
+          using namespace esdg_fx;
+          if (gen[el] == FX_NARROW) pass(std::integral_constant<int, FX_NARROW>{}, flat);
+          else if (gen[el] == FX_WIDE) pass(std::integral_constant<int, FX_WIDE>{}, flat);
+          else pass(std::integral_constant<int, FX_TALL>{}, flat);
+        };
+#ifdef FLAT_ALL
+        take(std::true_type{});
+#else
+        if (E2.sc.flat()) take(std::true_type{});
+        else take(std::false_type{});
+#endif
       } else {
         double acc[Nq][5];
 #pragma unroll
@@ -271,9 +282,8 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
         const double z0 = Z[0], z1 = Z[zs], z2 = Z[2 * zs];
         double r;
         if (!general) {
-          const int so = fxe[el2].out[v == 0 ? 0 : (v == 4 ? 2 : 1)];
           r = sJ * esdg_fx::from_fx(__double_as_longlong(z0) + __double_as_longlong(z1) +
-                                        __double_as_longlong(z2), so);
+                                        __double_as_longlong(z2), fxe[el2].out[v]);
           if (any_far) r = fma(sJ, far_terms<N>(g, a, e2, n, v, far_lift[el2]), r);
         } else {
           r = sJ * (z0 + z1 + z2);

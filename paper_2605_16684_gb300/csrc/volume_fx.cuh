@@ -7,11 +7,18 @@
 // instructions of a pair cost a warp 3900 cycles; the same pair in two-limb
 // fixed point, about 350 integer instructions, costs 640.  The node fields of
 // an element are scaled by powers of two to the element's own largest values
-// and held as value = h 2^30 + l, at least six bits finer than an FP64
-// significand at the largest value, and the pair pass runs on the integer
-// pipes.  Against the quad-precision sums of random pencils (N = 4) the error is
-// 0.25 to 0.42 of that of the FP64 pair in the series range and 1e-2 to 1e-6 of it
-// beyond.  Whole kernel, before (FP64 pairs) and after, one launch: 32^3 N = 4 warped bubble
+// and held as value = h 2^30 + l, and the pair pass runs on the integer pipes.
+//
+// A common scale holds a value of the largest size to 2^-59, six bits finer than an FP64
+// significand, and a smaller one to as many bits less as it is smaller.  What one sum adds
+// up therefore has to be of one size: the components of the metric and of the velocity
+// have a scale each, stretched against one another so that u_c Ja^d_c keeps its value
+// (metric_stretch).  With one scale for all, an element of 100 km x 100 km x 20 m lost
+// three digits of its horizontal fluxes.  Right-hand side without dissipation on boxes of
+// 1:1 to 1:1e5, N = 4, against long double: error over that of the FP64 pair 0.55 to 0.96
+// by variable.
+//
+// Whole kernel, before (FP64 pairs) and after, one launch: 32^3 N = 4 warped bubble
 // 3.400 -> 1.164 ms (narrow path), 16^3 N = 7 2.77 -> 0.79 ms, 16^3 N = 4 on a 2 km
 // box 0.494 -> 0.209 ms (wide path), 60 x 12 x 6 N = 4 channel 0.566 -> 0.233 ms
 // (tall path); with the launches of volume_fp64.cuh 0.973, 0.762 and 0.189 ms.
@@ -108,11 +115,14 @@ ESDG_HD unsigned hi32(unsigned a, unsigned b) { return (unsigned)(((u64)a * b) >
 struct FxScale {
   int ok;              // the element takes the fixed-point path
   int sr, sk, su, sn;  // density (halved), bracket and geopotential, velocity, metric
-  int s1;              // 2 su - sk - 60 >= 1: kinetic terms against the pressure terms
-  ESDG_HD int sp() const { return sr + sk - 60; }           // pressure
-  ESDG_HD int sF() const { return sr + su + sn - 121; }  // mass flux times Q
-  ESDG_HD int sM() const { return sp() + sn - 61; }      // momentum flux
-  ESDG_HD int sE() const { return sF() + sk - 60; }      // energy flux
+  int k[3];            // stretch of the components, the largest 0: u_c is held at su + k_c,
+                       // Ja^d_c at sn - k_c (metric_stretch)
+  ESDG_HD bool flat() const { return k[0] | k[1] | k[2]; }
+  int s1[3];           // 2 (su + k_c) - sk - 60 >= 1: kinetic terms against the pressure terms
+  ESDG_HD int sp() const { return sr + sk - 60; }                   // pressure
+  ESDG_HD int sF() const { return sr + su + sn - 121; }             // mass flux times Q
+  ESDG_HD int sM(int c) const { return sp() + sn - k[c] - 61; }     // momentum flux
+  ESDG_HD int sE() const { return sF() + sk - 60; }                 // energy flux
 };
 
 struct FxNode {  // rho/2, p/2, 1/(6 (gamma-1) b), ln(rho)/6, ln(b)/2, phi/2,
@@ -154,8 +164,8 @@ ESDG_HD Fx coth_poly(Fx y, Fx w) {
 // Wide: |y|, |dx| < 0.1225, polynomials fitted to 2^-55, the leading terms in two
 // limbs.  Tall: |dx| < 0.85.
 enum { FX_NARROW = 0, FX_WIDE = 1, FX_TALL = 2, FX_GENERAL = 3 };
-template <int PATH>
-ESDG_HD void pair_fx(const FxNode& A, const FxNode& B, Fx q, int s1, const Round& K, i64* ai,
+template <int PATH, bool FLAT>
+ESDG_HD void pair_fx(const FxNode& A, const FxNode& B, Fx q, const int* s1, const Round& K, i64* ai,
                      i64* al) {
   const Fx dy = A.y - B.y, dx = A.x - B.x;
   Fx fb, sg, ch, xx;
@@ -201,15 +211,18 @@ ESDG_HD void pair_fx(const FxNode& A, const FxNode& B, Fx q, int s1, const Round
   const Fx pt = (A.p + B.p) - limbs_b(mul(B.p - A.p, fb, K.l));
   const Fx pm = pt - V;
   // energy
-  const Fx br = (A.g + B.g) - limbs_b(mul(B.c - A.c, ch, K.l) -
-                                      (mul3(A.u0, B.u0, A.u1, B.u1, A.u2, B.u2, K.v) >> (s1 - 1)));
+  const i64 ke = FLAT ? (mul(A.u0, B.u0, K.v) >> (s1[0] - 1)) + (mul(A.u1, B.u1, K.v) >> (s1[1] - 1)) +
+                            (mul(A.u2, B.u2, K.v) >> (s1[2] - 1))
+                      : mul3(A.u0, B.u0, A.u1, B.u1, A.u2, B.u2, K.v) >> (s1[0] - 1);
+  const Fx br = (A.g + B.g) - limbs_b(mul(B.c - A.c, ch, K.l) - ke);
   const i64 E = mul2(limbs(F), br, pt, un, K.v);
   ai[4] += E;
   al[4] -= E;
   // momentum
-  const Fx Fs = limbs(F >> s1);
-  const i64 b0 = mul2(Fs, u0, pm, n0, K.v), b1 = mul2(Fs, u1, pm, n1, K.v),
-            b2 = mul2(Fs, u2, pm, n2, K.v);
+  const Fx F0 = limbs(F >> s1[0]), F1 = FLAT ? limbs(F >> s1[1]) : F0,
+           F2 = FLAT ? limbs(F >> s1[2]) : F0;
+  const i64 b0 = mul2(F0, u0, pm, n0, K.v), b1 = mul2(F1, u1, pm, n1, K.v),
+            b2 = mul2(F2, u2, pm, n2, K.v);
   const i64 g0 = mul(S, n0, K.v), g1 = mul(S, n1, K.v), g2 = mul(S, n2, K.v);
   ai[1] += b0 + g0;
   al[1] -= b0 - g0;
@@ -278,26 +291,41 @@ __device__ __forceinline__ void st_fx(double* p, Fx v) {
 }
 
 // An element's metric terms Ja/2 are kept in limbs (rows 0-8 of its geometry
-// block, 8 bytes each as the doubles they stand for) with their common scale
-// sn behind the last element's block; FX_NO_METRIC marks an element whose
+// block, 8 bytes each as the doubles they stand for) with the scales sn - k_c of their
+// three components behind the last element's block; FX_NO_METRIC marks an element whose
 // terms stay doubles (none or out of the sane range).
 constexpr int FX_NO_METRIC = -1000000;
 __host__ __device__ __forceinline__ int* metric_scales(const double* vgeo, size_t E, int np) {
   return const_cast<int*>(reinterpret_cast<const int*>(vgeo + E * ESDG_NVGEO * np));
 }
-// sn of an element whose largest squared norm of Ja^d/2 has this high word:
+// The stretch k_c <= 0 of the components from the high words of the largest |Ja^d_c/2|
+// of each: stretched to a common size, a flat element looks like a cube (u_c Ja^d_c, and
+// with it every mass flux, stays the same).  None where the largest terms of the
+// components lie within a factor of two to four: that costs at most two of the six
+// spare bits, and the pairs of an element without a stretch are 4 % cheaper (32^3 N = 4,
+// one launch: 0.987 against 1.022 ms; N = 7, 16^3: 0.752 and 0.777).
+__device__ __forceinline__ void metric_stretch(const unsigned* hi, int* k) {
+  const int e0 = (int)(hi[0] >> 20), e1 = (int)(hi[1] >> 20), e2 = (int)(hi[2] >> 20);
+  const int top = max(e0, max(e1, e2)), none = min(e0, min(e1, e2)) >= top - 1;
+  k[0] = none ? 0 : e0 - top;
+  k[1] = none ? 0 : e1 - top;
+  k[2] = none ? 0 : e2 - top;
+}
+// sn of an element whose largest squared norm of Ja^d/2 (stretched) has this high word:
 // the norm of Ja^d is below 2^(60 - sn)
-__device__ __forceinline__ int metric_scale(unsigned hi) {
+__device__ __forceinline__ int metric_scale(unsigned hi, const int* k) {
   const int e = (int)((hi >> 20) & 0x7ff) - 1022;  // |Ja^d/2|^2 < 2^e
-  return e > -240 && e < 240 ? 60 - (((e + 1) >> 1) + 1) : FX_NO_METRIC;
+  return e > -240 && e < 240 && min(k[0], min(k[1], k[2])) > -60 ? 60 - (((e + 1) >> 1) + 1)
+                                                                : FX_NO_METRIC;
 }
 
 // What a tile keeps per element: the scales, the first node's rho and 1/b
-// (the logarithms' reference), the scales of the three kinds of sums as they
-// leave the pencils, and the running maxima (high words) of the prologue.
+// (the logarithms' reference), the scales of the five sums as they leave the
+// pencils, and the running maxima (high words) of the prologue: the stretched
+// velocity's components and the geopotential.
 struct FxElement {
   FxScale sc;
-  int out[3];  // mass, momentum, energy
+  int out[5];
   unsigned mu, mf;
   double rq0, ib0;  // the first node's rho/4 and 1/b, as in log_ratio r0, b0,
   i64 r0, b0;
@@ -305,37 +333,58 @@ struct FxElement {
   int sb;           // scale of b0
 };
 
+// the stored scales of an element's metric, for its tile
+__device__ __forceinline__ void fx_metric(FxElement& E, const int* scales) {
+  const int s0 = scales[0], s1 = scales[1], s2 = scales[2];
+  E.sc.sn = min(s0, min(s1, s2));
+  E.sc.k[0] = E.sc.sn - s0;
+  E.sc.k[1] = E.sc.sn - s1;
+  E.sc.k[2] = E.sc.sn - s2;
+}
+// high word of |u 2^k|
+__device__ __forceinline__ unsigned stretched(double u, int k) {
+  return (unsigned)max((__double2hiint(u) & 0x7fffffff) + k * (1 << 20), 0);
+}
 // The scales of an element from its first node and the maxima; ok = 0 where a
 // field leaves the representation: a geopotential or kinetic energy far above
-// the internal energy, velocities near the speed of sound, gamma > 2.
-__device__ __forceinline__ void fx_scales(FxElement& E, double rq0, double ib0, int sn, double gm1,
+// the internal energy, velocities near the speed of sound (a stretched element:
+// the largest u_c Ja_c over the smallest Ja_c above a tenth of it), gamma > 2.
+__device__ __forceinline__ void fx_scales(FxElement& E, double rq0, double ib0, double gm1,
                                           double igm1, int wm) {
   auto expo = [](unsigned hi) { return (int)((hi >> 20) & 0x7ff) - 1022; };  // |v| < 2^expo
   auto sane = [&](unsigned hi) { return expo(hi) > -120 && expo(hi) < 120; };
   const unsigned hr = (unsigned)__double2hiint(rq0), hb = (unsigned)__double2hiint(ib0);
-  bool ok = !(hr >> 31) && !(hb >> 31) && sane(hr) && sane(hb) && sn != FX_NO_METRIC && gm1 <= 1.0 &&
-            expo(E.mu) < 60 && expo(E.mf) < 120;
+  FxScale s = E.sc;
+  const int eu = expo(E.mu) - min(s.k[0], min(s.k[1], s.k[2]));  // any velocity / 2 < 2^eu
+  bool ok = !(hr >> 31) && !(hb >> 31) && sane(hr) && sane(hb) && s.sn != FX_NO_METRIC && gm1 <= 1.0 &&
+            eu < 60 && expo(E.mf) < 120;
   // bracket: 1/(2 (gamma-1) b) (12 % above the first node's) + kinetic +
   // geopotential, below 2^(60 - sk)
-  const float um = ok ? __uint_as_float((unsigned)max(expo(E.mu) + 127, 1) << 23) : 1.0f;
+  const float um = ok ? __uint_as_float((unsigned)max(eu + 127, 1) << 23) : 1.0f;
   const float fm = ok ? __uint_as_float((unsigned)max(expo(E.mf) + 127, 1) << 23) : 1.0f;
-  const float k = ok ? fmaf(6.0f * um, um, fmaf(2.0f, fm, 0.565f * esdg_d2f(igm1 * ib0))) : 1.0f;
+  const float kin = 6.0f * um * um, rest = fmaf(2.0f, fm, 0.565f * esdg_d2f(igm1 * ib0));
+  const float k = ok ? kin + rest : 1.0f;
   const int eK = (int)((__float_as_uint(k) >> 23) & 0xff) - 126;
-  FxScale s;
   s.sr = 60 - (expo(hr) + 2);
   s.sk = 60 - eK;
-  // the norm of u, at most sqrt(3) times the largest component (u/2 in mu), is
-  // below 2^(60 - su)
+  // the norm of u (stretched), at most sqrt(3) times the largest component (u/2 in mu),
+  // is below 2^(60 - su)
   const int hm = (int)(E.mu & 0xfffffu) >= 0x279a7 ? 2 : 1;  // mantissa over 2/sqrt(3)
   s.su = 60 - max(expo(E.mu) + hm, -200);
-  s.sn = sn;
-  s.s1 = 2 * s.su - s.sk - 60;
-  s.ok = ok && s.s1 >= 1 && k < 1.0e30f;
-  s.s1 = min(s.s1, 63);
+  // Stretched, um is a bound that no node need come near, and what it takes from the
+  // pressure's and the small components' bits shows from um = 64 m/s on (1000 x 1000 x 10 m,
+  // u = 10, N = 4, error of rho u over that of the FP64 pairs: w = 0.5 0.81, w = 1 1.08,
+  // w = 2 1.22): 32 m/s at the temperature of air.
+  s.ok = ok && k < 1.0e30f && (!s.flat() || 16.0f * kin <= rest);
+  for (int c = 0; c < 3; c++) {
+    const int s1 = 2 * (s.su + s.k[c]) - s.sk - 60;
+    s.ok = s.ok && s1 >= 1;
+    s.s1[c] = min(s1, 63);
+    E.out[1 + c] = s.sM(c) - 2 - wm;
+  }
   E.sc = s;
   E.out[0] = s.sF() - 2 - wm;
-  E.out[1] = s.sM() - 2 - wm;
-  E.out[2] = s.sE() - 2 - wm;
+  E.out[4] = s.sE() - 2 - wm;
   E.rq0 = rq0;
   E.ib0 = ib0;
   E.sb = 59 - expo(hb);
@@ -391,7 +440,7 @@ __device__ __forceinline__ void fx_convert(double* S, int n, const FxElement& E,
   }
   st_fx(S + 2 * NP + n, to_fx(ib * (ce * (1.0 / 3.0)), s.sk));
 #pragma unroll
-  for (int k = 3; k < 6; k++) st_fx(S + k * NP + n, to_fx(S[k * NP + n], s.su));
+  for (int k = 3; k < 6; k++) st_fx(S + k * NP + n, to_fx(S[k * NP + n], s.su + s.k[k - 3]));
   const i64 f = to_fx64(S[6 * NP + n], s.sk);
   st_fx(S + 6 * NP + n, limbs(f));
   st_fx(S + 18 * NP + n, limbs(f + to_fx64(ib * (ce * 0.5), s.sk)));
