@@ -85,8 +85,8 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
       phantom = 0;
     }
     if (tid < EPB) {
-      if (tid < ne) esdg_fx::fx_metric(fxe[tid], nscale + 3 * (size_t)(e0 + tid));
-      fxe[tid].mu = fxe[tid].mf = 0u;
+      fxe[tid].mu = 0;
+      fxe[tid].mf = 0u;
       gen[tid] = 0u;
       for (int w = 0; w < 6; w++) far_lift[tid][w / 2][w % 2] = 0u;
     }
@@ -99,6 +99,7 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
       for (int k = 0; k < 9; k++) esdg_cp_async(S + (SH::F_NH + k) * NP, gr + k * NP);
       esdg_cp_async(S + 18 * NP, gr + 10 * NP);
     }
+    if (tid < ne) esdg_fx::fx_metric(fxe[tid], nscale + 3 * (size_t)(e0 + tid));
     esdg_cp_async_wait_all();  // these, and thread 0's edge elements of q
     const bool ok = tile_wait(&bar, parity);
     if (__syncthreads_or(!ok)) {
@@ -114,7 +115,7 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
         double* S = sm + (size_t)el * NF * NP;
         const double* qr = qr0 + (size_t)el * 5 * NP;
         prims64<NP>(qr[n], qr[NP + n], qr[2 * NP + n], qr[3 * NP + n], qr[4 * NP + n],
-                    S[18 * NP + n], gm1, S, n);
+                    S[18 * NP + n], S[18 * NP], gm1, S, n);
         const int* k = fxe[el].sc.k;
         using esdg_fx::stretched;
         atomicMax(&fxe[el].mu, max(stretched(S[3 * NP + n], k[0]), max(stretched(S[4 * NP + n], k[1]),
@@ -130,8 +131,9 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
       const unsigned path = esdg_fx::fx_path(S[n], S[2 * NP + n], S[0], S[2 * NP]);
       if (path != esdg_fx::FX_NARROW) atomicMax(&gen[el], path);
       if (n == 0) {
-        esdg_fx::fx_scales(fxe[el], S[0], S[2 * NP], P.gamma - 1.0, P.igm1, L.wm);
+        esdg_fx::fx_scales(fxe[el], S[0], S[2 * NP], S[18 * NP], P.gamma - 1.0, P.igm1, L.wm);
         if (!fxe[el].sc.ok) atomicMax(&gen[el], (unsigned)esdg_fx::FX_GENERAL);
+        else if (fxe[el].sc.tall()) atomicMax(&gen[el], (unsigned)esdg_fx::FX_TALL);
       }
     }
     __syncthreads();
@@ -158,12 +160,15 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
       // spare slots (mass, energy) as the nodes complete
       double* const om = S + (SH::F_NH + 3 * d) * NP + base;
       double* const ox = xs + ((size_t)el * 6 + 2 * d) * NP + base;
-      const FaceTerms<double> ft = face_fetch<N, double>(g, a, e0 + el, d, ps + Nq * pt);
+      FaceTerms<double> ft = face_fetch<N, double>(g, a, e0 + el, d, ps + Nq * pt);
       if (gen[el] != esdg_fx::FX_GENERAL) {
         using esdg_fx::i64;
         const esdg_fx::FxElement& E2 = fxe[el];
-        const int ks[3] = {E2.sc.s1[0], E2.sc.s1[1], E2.sc.s1[2]};
+        const int s1 = E2.sc.s1[0];
         i64 acc[Nq][5];
+        // energy fluxes relative to the element's geopotential (update restores it)
+        ft.m[4] = fma(-E2.phi0, ft.m[0], ft.m[4]);
+        ft.p[4] = fma(-E2.phi0, ft.p[0], ft.p[4]);
 #pragma unroll
         for (int v = 0; v < 5; v++) {
           const int so = E2.out[v];
@@ -191,27 +196,20 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
           om[NP + n] = out(2);
           om[2 * NP + n] = out(3);
         };
-        auto pass = [&](auto path, auto flat) {
+        auto pass = [&](auto path) {
           pencil_rolled<N>(acc, load,
                            [&](const esdg_fx::FxNode& A, const esdg_fx::FxNode& B, int i, int l,
                                i64* ai, i64* al) {
-                             esdg_fx::pair_fx<decltype(path)::value, decltype(flat)::value>(
-                                 A, B, esdg_fx::Fx{L.Qh[i][l], L.Ql[i][l]}, ks,
+                             const int* sp = decltype(path)::value == esdg_fx::FX_TALL ? E2.sc.s1 : &s1;
+                             esdg_fx::pair_fx<decltype(path)::value>(
+                                 A, B, esdg_fx::Fx{L.Qh[i][l], L.Ql[i][l]}, sp, E2.sc.dp,
                                  esdg_fx::Round{L.rnd[0], L.rnd[1]}, ai, al);
                            }, done);
         };
-        auto take = [&](auto flat) {
-          using namespace esdg_fx;
-          if (gen[el] == FX_NARROW) pass(std::integral_constant<int, FX_NARROW>{}, flat);
-          else if (gen[el] == FX_WIDE) pass(std::integral_constant<int, FX_WIDE>{}, flat);
-          else pass(std::integral_constant<int, FX_TALL>{}, flat);
-        };
-#ifdef FLAT_ALL
-        take(std::true_type{});
-#else
-        if (E2.sc.flat()) take(std::true_type{});
-        else take(std::false_type{});
-#endif
+        using namespace esdg_fx;
+        if (gen[el] == FX_NARROW) pass(std::integral_constant<int, FX_NARROW>{});
+        else if (gen[el] == FX_WIDE) pass(std::integral_constant<int, FX_WIDE>{});
+        else pass(std::integral_constant<int, FX_TALL>{});
       } else {
         double acc[Nq][5];
 #pragma unroll
@@ -273,6 +271,7 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
         f = P.f0 + P.beta * (o.y - P.y0);
         if (MODE != 0) f *= dt;
       }
+      double mass = 0.0;
 #pragma unroll
       for (int v = 0; v < 5; v++) {
         const bool mom = v >= 1 && v <= 3;
@@ -284,6 +283,8 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
         if (!general) {
           r = sJ * esdg_fx::from_fx(__double_as_longlong(z0) + __double_as_longlong(z1) +
                                         __double_as_longlong(z2), fxe[el2].out[v]);
+          if (v == 0) mass = r;
+          if (v == 4) r = fma(fxe[el2].phi0, mass, r);
           if (any_far) r = fma(sJ, far_terms<N>(g, a, e2, n, v, far_lift[el2]), r);
         } else {
           r = sJ * (z0 + z1 + z2);

@@ -14,9 +14,14 @@
 // up therefore has to be of one size: the components of the metric and of the velocity
 // have a scale each, stretched against one another so that u_c Ja^d_c keeps its value
 // (metric_stretch).  With one scale for all, an element of 100 km x 100 km x 20 m lost
-// three digits of its horizontal fluxes.  Right-hand side without dissipation on boxes of
-// 1:1 to 1:1e5, N = 4, against long double: error over that of the FP64 pair 0.55 to 0.96
-// by variable.
+// three digits of its horizontal fluxes.  The geopotential is relative to the element's
+// first node (the energy's interface terms as well; the kernel restores it from the mass
+// sum), and the pressure's scale stands above the energies' where they are much larger
+// (FxScale::dp): gamma near 1 and meshes far above z = 0 lost up to five bits of it.
+// Right-hand side without dissipation against long double, error over that of the FP64
+// pair by variable, N = 2 to 7: cubes at rest to 100 m/s 0.4 to 0.95, boxes of 1:1 to 1:1e5
+// 0.4 to 0.96, elements of 3 to 11 km 0.4 to 1.0, gamma 1.05 to 2 0.45 to 0.95; N = 1 up to
+// 1.1.
 //
 // Whole kernel, before (FP64 pairs) and after, one launch: 32^3 N = 4 warped bubble
 // 3.400 -> 1.164 ms (narrow path), 16^3 N = 7 2.77 -> 0.79 ms, 16^3 N = 4 on a 2 km
@@ -27,9 +32,10 @@
 // result does not depend on the tile: all densities and 1/b = 2p/rho positive and
 // within 0.95 % (narrow) or 12 % (wide) of the first node's, or densities between
 // 0.21 and 1.12 of it (tall: a stratified element whose first node is its
-// lowest); metric terms and geopotential in a sane range, gamma <= 2, kinetic
-// energy below a quarter of the internal plus potential energy.  The lines lie
-// where the correction series leave 2^-51 (narrow), 2^-55 (wide, tall); all other
+// lowest); metric terms in a sane range, gamma <= 2, velocities
+// up to about half the speed of sound.  An element whose internal energy or geopotential
+// difference is well above p/rho takes the tall path too, which gives the pressure a
+// scale of its own.  The lines lie where the correction series leave 2^-51 (narrow), 2^-55 (wide, tall); all other
 // elements take pair64.  The wide path costs a pair about 900 cycles, the tall one
 // 1000.
 //
@@ -117,15 +123,17 @@ struct FxScale {
   int sr, sk, su, sn;  // density (halved), bracket and geopotential, velocity, metric
   int k[3];            // stretch of the components, the largest 0: u_c is held at su + k_c,
                        // Ja^d_c at sn - k_c (metric_stretch)
-  ESDG_HD bool flat() const { return k[0] | k[1] | k[2]; }
-  int s1[3];           // 2 (su + k_c) - sk - 60 >= 1: kinetic terms against the pressure terms
-  ESDG_HD int sp() const { return sr + sk - 60; }                   // pressure
+  ESDG_HD bool flat() const { return k[0] + k[1] + k[2] < 0; }
+  ESDG_HD bool tall() const { return flat() || dp; }  // only the tall path has such scales
+  int dp;              // bits by which the pressure's scale is above the bracket's
+  int s1[3];           // 2 (su + k_c) - sk - dp - 60 >= 1: kinetic terms against the pressure terms
+  ESDG_HD int sp() const { return sr + sk + dp - 60; }              // pressure
   ESDG_HD int sF() const { return sr + su + sn - 121; }             // mass flux times Q
   ESDG_HD int sM(int c) const { return sp() + sn - k[c] - 61; }     // momentum flux
   ESDG_HD int sE() const { return sF() + sk - 60; }                 // energy flux
 };
 
-struct FxNode {  // rho/2, p/2, 1/(6 (gamma-1) b), ln(rho)/6, ln(b)/2, phi/2,
+struct FxNode {  // rho/2, p/2, 1/(6 (gamma-1) b), ln(rho)/6, ln(b)/2, phi/2 (at sk + dp),
                  // phi/2 + 1/(4 (gamma-1) b), u/2, Ja^d/2
   Fx r, p, c, x, y, f, g, u0, u1, u2, n0, n1, n2;
 };
@@ -162,11 +170,14 @@ ESDG_HD Fx coth_poly(Fx y, Fx w) {
 // Narrow: each is the difference plus its cube times a linear polynomial in its
 // square, in 30 bits (|y| < 0.0098; what is left out stays below 2^-51).
 // Wide: |y|, |dx| < 0.1225, polynomials fitted to 2^-55, the leading terms in two
-// limbs.  Tall: |dx| < 0.85.
+// limbs.  Tall: |dx| < 0.85, and any scales: components stretched against one another
+// (s1 by component), the pressure's above the bracket's (dp).
 enum { FX_NARROW = 0, FX_WIDE = 1, FX_TALL = 2, FX_GENERAL = 3 };
-template <int PATH, bool FLAT>
-ESDG_HD void pair_fx(const FxNode& A, const FxNode& B, Fx q, const int* s1, const Round& K, i64* ai,
-                     i64* al) {
+template <int PATH>
+ESDG_HD void pair_fx(const FxNode& A, const FxNode& B, Fx q, const int* s1, int dp, const Round& K,
+                     i64* ai, i64* al) {
+  constexpr bool TALL = PATH == FX_TALL;
+  if (!TALL) dp = 0;
   const Fx dy = A.y - B.y, dx = A.x - B.x;
   Fx fb, sg, ch, xx;
   if (PATH != FX_NARROW) {
@@ -211,16 +222,18 @@ ESDG_HD void pair_fx(const FxNode& A, const FxNode& B, Fx q, const int* s1, cons
   const Fx pt = (A.p + B.p) - limbs_b(mul(B.p - A.p, fb, K.l));
   const Fx pm = pt - V;
   // energy
-  const i64 ke = FLAT ? (mul(A.u0, B.u0, K.v) >> (s1[0] - 1)) + (mul(A.u1, B.u1, K.v) >> (s1[1] - 1)) +
-                            (mul(A.u2, B.u2, K.v) >> (s1[2] - 1))
-                      : mul3(A.u0, B.u0, A.u1, B.u1, A.u2, B.u2, K.v) >> (s1[0] - 1);
+  const int t = dp - 1;
+  const i64 ke = TALL ? (mul(A.u0, B.u0, K.v) >> (s1[0] + t)) + (mul(A.u1, B.u1, K.v) >> (s1[1] + t)) +
+                            (mul(A.u2, B.u2, K.v) >> (s1[2] + t))
+                      : mul3(A.u0, B.u0, A.u1, B.u1, A.u2, B.u2, K.v) >> (s1[0] + t);
   const Fx br = (A.g + B.g) - limbs_b(mul(B.c - A.c, ch, K.l) - ke);
-  const i64 E = mul2(limbs(F), br, pt, un, K.v);
+  const i64 E = TALL ? mul(limbs(F), br, K.v) + (mul(pt, un, K.v) >> dp)
+                     : mul2(limbs(F), br, pt, un, K.v);
   ai[4] += E;
   al[4] -= E;
   // momentum
-  const Fx F0 = limbs(F >> s1[0]), F1 = FLAT ? limbs(F >> s1[1]) : F0,
-           F2 = FLAT ? limbs(F >> s1[2]) : F0;
+  const Fx F0 = limbs(F >> s1[0]), F1 = TALL ? limbs(F >> s1[1]) : F0,
+           F2 = TALL ? limbs(F >> s1[2]) : F0;
   const i64 b0 = mul2(F0, u0, pm, n0, K.v), b1 = mul2(F1, u1, pm, n1, K.v),
             b2 = mul2(F2, u2, pm, n2, K.v);
   const i64 g0 = mul(S, n0, K.v), g1 = mul(S, n1, K.v), g2 = mul(S, n2, K.v);
@@ -276,7 +289,9 @@ __device__ __forceinline__ Fx to_fx(double v, int s) { return limbs(to_fx64(v, s
 // infinite one has no exponent to add to.
 __device__ __forceinline__ double from_fx(i64 v, int s) {
   const double d = (double)v;
-  return __hiloint2double(v ? __double2hiint(d) - s * (1 << 20) : 0, __double2loint(d));
+  int hi = __double2hiint(d);
+  if (hi) hi -= s * (1 << 20);
+  return __hiloint2double(hi, __double2loint(d));
 }
 // does v 2^s leave the limbs' range by 2^-b? (infinities and NaNs do)
 __device__ __forceinline__ bool fx_over(double v, int s, int b) {
@@ -302,8 +317,7 @@ __host__ __device__ __forceinline__ int* metric_scales(const double* vgeo, size_
 // of each: stretched to a common size, a flat element looks like a cube (u_c Ja^d_c, and
 // with it every mass flux, stays the same).  None where the largest terms of the
 // components lie within a factor of two to four: that costs at most two of the six
-// spare bits, and the pairs of an element without a stretch are 4 % cheaper (32^3 N = 4,
-// one launch: 0.987 against 1.022 ms; N = 7, 16^3: 0.752 and 0.777).
+// spare bits and keeps the element off the tall path.
 __device__ __forceinline__ void metric_stretch(const unsigned* hi, int* k) {
   const int e0 = (int)(hi[0] >> 20), e1 = (int)(hi[1] >> 20), e2 = (int)(hi[2] >> 20);
   const int top = max(e0, max(e1, e2)), none = min(e0, min(e1, e2)) >= top - 1;
@@ -326,11 +340,13 @@ __device__ __forceinline__ int metric_scale(unsigned hi, const int* k) {
 struct FxElement {
   FxScale sc;
   int out[5];
-  unsigned mu, mf;
+  int mu;
+  unsigned mf;
   double rq0, ib0;  // the first node's rho/4 and 1/b, as in log_ratio r0, b0,
   i64 r0, b0;
   Fx ir0, inb0;     // and their reciprocals
   int sb;           // scale of b0
+  double phi0;      // the first node's geopotential: the pairs' is relative to it
 };
 
 // the stored scales of an element's metric, for its tile
@@ -341,21 +357,22 @@ __device__ __forceinline__ void fx_metric(FxElement& E, const int* scales) {
   E.sc.k[1] = E.sc.sn - s1;
   E.sc.k[2] = E.sc.sn - s2;
 }
-// high word of |u 2^k|
-__device__ __forceinline__ unsigned stretched(double u, int k) {
-  return (unsigned)max((__double2hiint(u) & 0x7fffffff) + k * (1 << 20), 0);
+// high word of |u 2^k|, not positive where that is too small to matter
+__device__ __forceinline__ int stretched(double u, int k) {
+  return (__double2hiint(u) & 0x7fffffff) + k * (1 << 20);
 }
 // The scales of an element from its first node and the maxima; ok = 0 where a
-// field leaves the representation: a geopotential or kinetic energy far above
-// the internal energy, velocities near the speed of sound (a stretched element:
-// the largest u_c Ja_c over the smallest Ja_c above a tenth of it), gamma > 2.
-__device__ __forceinline__ void fx_scales(FxElement& E, double rq0, double ib0, double gm1,
-                                          double igm1, int wm) {
+// field leaves the representation or loses more than the spare bits: velocities of about
+// half the speed of sound (a stretched element: the largest u_c Ja_c over the smallest
+// Ja_c above a tenth of it), gamma > 2 or below 1.005, geopotential differences above the
+// energies.
+__device__ __forceinline__ void fx_scales(FxElement& E, double rq0, double ib0, double phi0,
+                                          double gm1, double igm1, int wm) {
   auto expo = [](unsigned hi) { return (int)((hi >> 20) & 0x7ff) - 1022; };  // |v| < 2^expo
   auto sane = [&](unsigned hi) { return expo(hi) > -120 && expo(hi) < 120; };
   const unsigned hr = (unsigned)__double2hiint(rq0), hb = (unsigned)__double2hiint(ib0);
   FxScale s = E.sc;
-  const int eu = expo(E.mu) - min(s.k[0], min(s.k[1], s.k[2]));  // any velocity / 2 < 2^eu
+  const int low = min(s.k[0], min(s.k[1], s.k[2])), eu = expo(E.mu) - low;  // any velocity / 2 < 2^eu
   bool ok = !(hr >> 31) && !(hb >> 31) && sane(hr) && sane(hb) && s.sn != FX_NO_METRIC && gm1 <= 1.0 &&
             eu < 60 && expo(E.mf) < 120;
   // bracket: 1/(2 (gamma-1) b) (12 % above the first node's) + kinetic +
@@ -365,6 +382,10 @@ __device__ __forceinline__ void fx_scales(FxElement& E, double rq0, double ib0, 
   const float kin = 6.0f * um * um, rest = fmaf(2.0f, fm, 0.565f * esdg_d2f(igm1 * ib0));
   const float k = ok ? kin + rest : 1.0f;
   const int eK = (int)((__float_as_uint(k) >> 23) & 0xff) - 126;
+  // The pressure p = rho / (2b) is held at the bracket's scale while that is below 3/b
+  // (gamma = 1.4 at rest: 1.4 to 2.8, by the power of two); above, its scale is raised by
+  // as many bits, on the tall path.
+  s.dp = max(eK - ((int)(__float_as_uint(3.0f * esdg_d2f(ib0)) >> 23) - 127), 0);
   s.sr = 60 - (expo(hr) + 2);
   s.sk = 60 - eK;
   // the norm of u (stretched), at most sqrt(3) times the largest component (u/2 in mu),
@@ -375,17 +396,18 @@ __device__ __forceinline__ void fx_scales(FxElement& E, double rq0, double ib0, 
   // pressure's and the small components' bits shows from um = 64 m/s on (1000 x 1000 x 10 m,
   // u = 10, N = 4, error of rho u over that of the FP64 pairs: w = 0.5 0.81, w = 1 1.08,
   // w = 2 1.22): 32 m/s at the temperature of air.
-  s.ok = ok && k < 1.0e30f && (!s.flat() || 16.0f * kin <= rest);
+  s.ok = ok && k < 1.0e30f && s.dp < 8 && expo(E.mf) + 1 + s.dp <= eK && (!s.flat() || 16.0f * kin <= rest);
+  const int s1 = 2 * s.su - s.sk - s.dp - 60;
+  s.ok = s.ok && s1 + 2 * low >= 1;
   for (int c = 0; c < 3; c++) {
-    const int s1 = 2 * (s.su + s.k[c]) - s.sk - 60;
-    s.ok = s.ok && s1 >= 1;
-    s.s1[c] = min(s1, 63);
+    s.s1[c] = min(s1 + 2 * s.k[c], 55);  // a shift of s1 + dp stays below 64
     E.out[1 + c] = s.sM(c) - 2 - wm;
   }
   E.sc = s;
   E.out[0] = s.sF() - 2 - wm;
   E.out[4] = s.sE() - 2 - wm;
   E.rq0 = rq0;
+  E.phi0 = phi0;
   E.ib0 = ib0;
   E.sb = 59 - expo(hb);
   if (s.ok) {
@@ -441,9 +463,9 @@ __device__ __forceinline__ void fx_convert(double* S, int n, const FxElement& E,
   st_fx(S + 2 * NP + n, to_fx(ib * (ce * (1.0 / 3.0)), s.sk));
 #pragma unroll
   for (int k = 3; k < 6; k++) st_fx(S + k * NP + n, to_fx(S[k * NP + n], s.su + s.k[k - 3]));
-  const i64 f = to_fx64(S[6 * NP + n], s.sk);
+  const i64 f = to_fx64(S[6 * NP + n], s.sk + s.dp);
   st_fx(S + 6 * NP + n, limbs(f));
-  st_fx(S + 18 * NP + n, limbs(f + to_fx64(ib * (ce * 0.5), s.sk)));
+  st_fx(S + 18 * NP + n, limbs((f >> s.dp) + to_fx64(ib * (ce * 0.5), s.sk)));
   st_fx(S + 8 * NP + n, to_fx(ph, s.sp()));
 }
 

@@ -522,11 +522,12 @@ __device__ double far_terms(const EsdgGrid& g, const EsdgVolArgs& a, int e, int 
   return sum;
 }
 // FP64 node primitives from the conserved state: rho/4, 1/b = 2p/rho, u/2,
-// phi/2 and p/2 (in the slot of ln b), with p = (gamma - 1)(E - rho phi -
-// |rho u|^2/(2 rho)).  b/2 and the logarithms follow in prims64_general for the elements that need them.
+// phi/2 relative to the element's first node (phi0) and p/2 (in the slot of ln b), with
+// p = (gamma - 1)(E - rho phi - |rho u|^2/(2 rho)).  b/2, the logarithms and the whole
+// phi/2 follow in prims64_general for the elements that need them.
 template <int NP>
 __device__ __forceinline__ void prims64(double q0, double q1, double q2, double q3, double q4,
-                                        double phi, double gm1, double* S, int n) {
+                                        double phi, double phi0, double gm1, double* S, int n) {
   const double ir = esdg_rcp(q0);
   const double hi = esdg_ldexp(ir, -1);
   const double u0 = q1 * hi, u1 = q2 * hi, u2 = q3 * hi;
@@ -540,17 +541,18 @@ __device__ __forceinline__ void prims64(double q0, double q1, double q2, double 
   S[3 * NP + n] = u0;
   S[4 * NP + n] = u1;
   S[5 * NP + n] = u2;
-  S[6 * NP + n] = 0.5 * phi;
+  S[6 * NP + n] = fma(0.5, phi, -esdg_ldexp(phi0, -1));
   S[8 * NP + n] = ph;
 }
-// the remaining fields of pair64: b/2 = 1/(2 (1/b)), ln rho, ln b, and Ja/2
-// (Ja: the element's [3][3][NP] block)
+// the remaining fields of pair64: b/2 = 1/(2 (1/b)), phi/2 (phi in the spare field),
+// ln rho, ln b, and Ja/2 (Ja: the element's [3][3][NP] block)
 template <int NP>
 __device__ __forceinline__ void prims64_general(double* S, int n, const double* Ja) {
 #pragma unroll
   for (int k = 0; k < 9; k++) S[(9 + k) * NP + n] = esdg_ldexp(Ja[k * NP + n], -1);
   const double bh = esdg_ldexp(esdg_rcp(S[2 * NP + n]), -1);
   S[1 * NP + n] = bh;
+  S[6 * NP + n] = 0.5 * S[18 * NP + n];
   S[7 * NP + n] = log(4.0 * S[n]);
   S[8 * NP + n] = log(2.0 * bh);
 }
