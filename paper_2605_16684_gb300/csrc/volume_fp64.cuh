@@ -57,6 +57,7 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
   // per element: its path; the pencils (three directions, 64
   // bits) whose interface terms leave its range
   __shared__ unsigned gen[EPB], far_lift[EPB][3][2];
+  __shared__ bool logs[EPB];  // a node outside the narrow path's range
   double* const sm = reinterpret_cast<double*>(smraw) + F64<N>::S0;
   double* const xs = reinterpret_cast<double*>(smraw) + F64<N>::X0;
   const int tid = threadIdx.x;
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
       fxe[tid].mu = 0;
       fxe[tid].mf = 0u;
       gen[tid] = 0u;
+      logs[tid] = false;
       for (int w = 0; w < 6; w++) far_lift[tid][w / 2][w % 2] = 0u;
     }
     // the metric limbs and (in the spare field) the geopotential
@@ -129,7 +131,10 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
       const int el = idx / NP, n = idx - el * NP;
       const double* S = sm + (size_t)el * NF * NP;
       const unsigned path = esdg_fx::fx_path(S[n], S[2 * NP + n], S[0], S[2 * NP]);
-      if (path != esdg_fx::FX_NARROW) atomicMax(&gen[el], path);
+      if (path != esdg_fx::FX_NARROW) {
+        atomicMax(&gen[el], path);
+        logs[el] = true;
+      }
       if (n == 0) {
         esdg_fx::fx_scales(fxe[el], S[0], S[2 * NP], S[18 * NP], P.gamma - 1.0, P.igm1, L.wm);
         if (!fxe[el].sc.ok) atomicMax(&gen[el], (unsigned)esdg_fx::FX_GENERAL);
@@ -140,7 +145,8 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
     for (int idx = tid; idx < ne * NP; idx += T) {
       const int el = idx / NP, n = idx - el * NP;
       double* S = sm + (size_t)el * NF * NP;
-      if (gen[el] == esdg_fx::FX_GENERAL) prims64_general<NP>(S, n, a.Ja + (size_t)(e0 + el) * 9 * NP);
+      if (gen[el] == esdg_fx::FX_GENERAL)
+        prims64_general<NP>(S, n, a.Ja + (size_t)(e0 + el) * 9 * NP, logs[el]);
       else esdg_fx::fx_convert<NP>(S, n, fxe[el], gen[el], 0.5 * P.igm1);
     }
     __syncthreads();
@@ -217,11 +223,14 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
 #pragma unroll
           for (int v = 0; v < 5; v++) acc[i][v] = i == 0 ? -ft.m[v] : (i == N ? ft.p[v] : 0.0);
         const CeSeries cs = ce_series(0.5 * P.igm1);
-        pencil_rolled<N>(
+        // unrolled: independent pairs side by side, as the FP64 pipe's latency needs (rolled,
+        // 24^3 N = 4 and 14^3 N = 7 at Mach 1, one right-hand side: 1.720 and 2.113 ms
+        // against 1.666 and 1.995)
+        pencil_unrolled<N>(
             acc,
             [&](int i) { return load_node<double, true, SH::F_NH, NP, 0>(S, base + i * stride, d); },
             [&](const Node<double>& A, const Node<double>& B, int i, int l, double* ai, double* al) {
-              pair64<true>(A, B, L.Dt[i][l], L.Dt[l][i], cs, ai, al);
+              pair64(A, B, L.Dt[i][l], L.Dt[l][i], cs, ai, al);
             },
             [&](int i, const double* s) {
               const int n = i * stride;

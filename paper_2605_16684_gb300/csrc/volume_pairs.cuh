@@ -98,7 +98,6 @@ __device__ __forceinline__ double esdg_Ace_t(double u, const CeSeries& c) {
 // series path.  ai += Dt_il H(i,l), al += Dt_li H(l,i).  The momentum flux is
 // regrouped as Fr {{u}} + (p* + g_own) {{n}}, so the gravity coefficient of
 // each side folds into its pressure term with one FMA.
-template <bool LOGS>
 __device__ __forceinline__ void pair64(const Node<double>& A, const Node<double>& B, double dil,
                                        double dli, const CeSeries& cs, double* ai, double* al) {
   const double sr = A.rq + B.rq;  // {{rho}}/2
@@ -111,15 +110,10 @@ __device__ __forceinline__ void pair64(const Node<double>& A, const Node<double>
   const double uu = fma(A.u2, B.u2, fma(A.u1, B.u1, A.u0 * B.u0));  // u_i . u_l / 4
   const double t = fma(2.0, uu, A.ph + B.ph);                        // u_i.u_l/2 + {{phi}}
   double rlog, bracket;  // <rho>_log and ce/<b>_log + t
-  if (!LOGS) {
-    rlog = sr * esdg_Q2_t(ur);
-    bracket = fma(rsb, esdg_Ace_t(ub, cs), t);
-  } else {
-    if (esdg_lt_pos(ur, ESDG_LOG_EPS)) rlog = sr * esdg_Q2_t(ur);
-    else rlog = (4.0 * dr) * esdg_rcp(A.lr - B.lr);
-    if (esdg_lt_pos(ub, ESDG_LOG_EPS)) bracket = fma(rsb, esdg_Ace_t(ub, cs), t);
-    else bracket = fma((A.lb - B.lb) * esdg_rcp(2.0 * db), cs.c0, t);
-  }
+  if (esdg_lt_pos(ur, ESDG_LOG_EPS)) rlog = sr * esdg_Q2_t(ur);
+  else rlog = (4.0 * dr) * esdg_rcp(A.lr - B.lr);
+  if (esdg_lt_pos(ub, ESDG_LOG_EPS)) bracket = fma(rsb, esdg_Ace_t(ub, cs), t);
+  else bracket = fma((A.lb - B.lb) * esdg_rcp(2.0 * db), cs.c0, t);
   const double n0 = A.n0 + B.n0, n1 = A.n1 + B.n1, n2 = A.n2 + B.n2;  // {{Ja^d}}
   const double u0 = A.u0 + B.u0, u1 = A.u1 + B.u1, u2 = A.u2 + B.u2;  // {{u}}
   const double un = fma(u2, n2, fma(u1, n1, u0 * n0));
@@ -545,14 +539,16 @@ __device__ __forceinline__ void prims64(double q0, double q1, double q2, double 
   S[8 * NP + n] = ph;
 }
 // the remaining fields of pair64: b/2 = 1/(2 (1/b)), phi/2 (phi in the spare field),
-// ln rho, ln b, and Ja/2 (Ja: the element's [3][3][NP] block)
+// Ja/2 (Ja: the element's [3][3][NP] block) and ln rho, ln b (logs: some pair may leave the
+// series range; the pairs of the others do not use them)
 template <int NP>
-__device__ __forceinline__ void prims64_general(double* S, int n, const double* Ja) {
+__device__ __forceinline__ void prims64_general(double* S, int n, const double* Ja, bool logs) {
 #pragma unroll
   for (int k = 0; k < 9; k++) S[(9 + k) * NP + n] = esdg_ldexp(Ja[k * NP + n], -1);
   const double bh = esdg_ldexp(esdg_rcp(S[2 * NP + n]), -1);
   S[1 * NP + n] = bh;
   S[6 * NP + n] = 0.5 * S[18 * NP + n];
+  if (!logs) return;
   S[7 * NP + n] = log(4.0 * S[n]);
   S[8 * NP + n] = log(2.0 * bh);
 }
