@@ -169,18 +169,21 @@ __device__ __forceinline__ double esdg_ldexp(double x, int k) {
   return __hiloint2double(hi + k * (1 << 20), __double2loint(x));
 }
 
-// ---- launches that start while the launch before them in the stream still runs
-// Device: wait until that launch is complete and its writes are visible, then let
-// the launch after this one start in the same way.  First in every kernel that
-// esdg_launch starts, before any access to memory; without `after` it is a no-op.
+// ---- launches that start while the launch before them in the stream ends
+// Device: wait until that launch is complete and its writes are visible.  First in
+// every kernel that esdg_launch starts, before any access to memory; without `after`
+// it is a no-op.  No kernel lets the next launch start before its own CTAs have ended
+// (griddepcontrol.launch_dependents): CTAs of the next launch that are placed while this
+// one's hold the SMs pile up on some of them, and a launch of up to a few CTAs per SM
+// waits for the fullest.  One LSRK step, us: started early / as here / plain launches:
+// mixed 4^3 N = 7 180 / 108 / 134, 8^3 N = 4 98 / 73 / 93; FP64 4^3 N = 3 127 / 128 / 151,
+// 6^3 N = 5 361 / 260 / 287, 8^3 N = 4 363 / 270 / 288; from 10^3 N = 6 on alike.
 __device__ __forceinline__ void esdg_wait_before() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 // Host: launch k; after != 0 only when the launch before it in the stream is one of
-// this library's that calls esdg_wait_before (the stages of a step): its CTAs are then
-// resident and waiting when that launch ends.  One LSRK step of ten launches: mixed
-// 80x16x8 N = 3 471 -> 452 us, mixed 8^3 N = 4 120 -> 107 us, FP64 4^3 N = 3 177 -> 155 us.
+// this library's that calls esdg_wait_before (the stages of a step): it is then set up
+// while that launch ends.
 template <typename... P, typename... A>
 cudaError_t esdg_launch(void (*k)(P...), int after, unsigned grid, unsigned block, size_t smem,
                         cudaStream_t s, A&&... args) {
