@@ -22,6 +22,9 @@ const double kRkB[5] = {1432997174477.0 / 9575080441755.0, 5161836677717.0 / 136
                         1720146321549.0 / 2090206949498.0, 3134564353537.0 / 4481467310338.0,
                         2277821191437.0 / 14882151754819.0};
 
+// set when a bounded wait of a volume kernel ran out; read and cleared by es_dg_sync
+__device__ int g_wait_timeout;
+
 }  // namespace
 
 struct es_dg {
@@ -45,6 +48,7 @@ struct es_dg {
   double* result;   // small device result slots (3 doubles, then the status word)
   int* status;      // set by a stage update whose new state is not finite or has a
                     // non-positive density; read and cleared by es_dg_sync
+  int* timeout;     // g_wait_timeout on the handle's device
   // mixed precision relative to a hydrostatic background
   int has_bg;
   double* bg;       // [E][3][np] rho_bg, b_bg, p_bg
@@ -195,6 +199,7 @@ EsdgVolArgs vol_args(es_dg_t* h, const double* q_in, double* rhs_out) {
   a.rkB = 0.0;
   a.dt = 0.0;
   a.status = h->status;
+  a.timeout = h->timeout;
   a.share = 1;
   a.after = 0;
   return a;
@@ -513,7 +518,8 @@ int create_impl(const es_dg_mesh* mesh, int N, es_dg_precision precision,
     return st;
   }
   h->status = reinterpret_cast<int*>(h->result + 3);
-  cudaError_t e = cudaMemsetAsync(h->result, 0, 4 * sizeof(double), h->stream);
+  cudaError_t e = cudaGetSymbolAddress(reinterpret_cast<void**>(&h->timeout), g_wait_timeout);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->result, 0, 4 * sizeof(double), h->stream);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(h->dq, 0, nq * (h->mixed ? sizeof(float) : sizeof(double)), h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->q, 0, nq * sizeof(double), h->stream);
@@ -766,13 +772,21 @@ int es_dg_sync(es_dg_t* h) {
   if (!h) return ES_DG_EINVAL;
   const int st = cuda_status(cudaStreamSynchronize(h->stream));
   if (st != ES_DG_OK) return st;
-  const int t64 = esdg_volume_f64_take_timeout(), t32 = esdg_volume_mixed_take_timeout(),
-            t32o = esdg_volume_mixed_other_take_timeout();
-  if (t64 < 0 || t32 < 0 || t32o < 0) return ES_DG_ECUDA;
-  if (t64 || t32 || t32o) return ES_DG_ETIMEOUT;
-  const int bad = esdg_take_status(h);
-  if (bad < 0) return ES_DG_ECUDA;
-  return bad ? ES_DG_ENAN : ES_DG_OK;
+  // both words in one go (each copy and its wait take some 8 us)
+  int late = 0, bad = 0;
+  cudaError_t e = cudaMemcpyAsync(&late, h->timeout, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(&bad, h->status, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess && (late || bad)) {  // a timeout is reported first, alone
+    e = cudaMemsetAsync(late ? h->timeout : h->status, 0, sizeof(int), h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return ES_DG_ECUDA;
+  }
+  return late ? ES_DG_ETIMEOUT : bad ? ES_DG_ENAN : ES_DG_OK;
 }
 
 int es_dg_integrals(es_dg_t* h, double out[3]) {

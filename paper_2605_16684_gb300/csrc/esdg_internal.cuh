@@ -391,6 +391,7 @@ struct EsdgVolArgs {
   double rkA, rkB, dt;
   int* status;           // mode 1: set to 1 when an updated state value is not finite or a
                          // density is not positive (null: not checked)
+  int* timeout;          // set to 1 when a bounded wait of the kernel ran out (one word per device)
   int share;             // launches of this kind that run side by side (slabs of one mesh)
   int after;             // the launch before this one in the stream is the stage's interface kernel
 };
@@ -428,11 +429,6 @@ int esdg_volume_batch_variants_mixed(int N);
 // volume launch registers on its first barrier without copying them;
 // read and cleared by the launcher.
 unsigned esdg_take_phantom();
-// 1 if a bounded wait of the FP64 / mixed volume kernels ran out
-// since the last call (the flag is cleared), 0 if not, -1 on a CUDA error
-int esdg_volume_f64_take_timeout();
-int esdg_volume_mixed_take_timeout();
-int esdg_volume_mixed_other_take_timeout();
 cudaError_t esdg_launch_volume_f64(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys& P, int mode,
                                    const EsdgVolArgs& a, cudaStream_t s);
 cudaError_t esdg_launch_volume_mixed(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys& P,

@@ -4,8 +4,6 @@
 #include "volume_impl.cuh"
 #include "volume_mixed.cuh"
 
-int esdg_volume_mixed_take_timeout() { return esdg_vol::take_timeout(); }
-
 cudaError_t esdg_launch_volume_mixed(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys& P,
                                      int mode, const EsdgVolArgs& a, cudaStream_t s) {
   if (!a.bg || a.bgq) return esdg_launch_volume_mixed_other(g, L, P, mode, a, s);

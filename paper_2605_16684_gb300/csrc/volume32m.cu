@@ -5,8 +5,6 @@
 #include "volume_impl.cuh"
 #include "volume_mixed.cuh"
 
-int esdg_volume_mixed_other_take_timeout() { return esdg_vol::take_timeout(); }
-
 cudaError_t esdg_launch_volume_mixed_other(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys& P,
                                            int mode, const EsdgVolArgs& a, cudaStream_t s) {
   using namespace esdg_vol;

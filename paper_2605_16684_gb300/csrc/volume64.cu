@@ -3,8 +3,6 @@
 #include "volume_fp64.cuh"
 #include "volume_impl.cuh"
 
-int esdg_volume_f64_take_timeout() { return esdg_vol::take_timeout(); }
-
 cudaError_t esdg_launch_volume_f64(const EsdgGrid& g, const EsdgLGL& L, const EsdgPhys& P, int mode,
                                    const EsdgVolArgs& a, cudaStream_t s) {
   return esdg_vol::for_order(g.N, cudaErrorInvalidValue, [&](auto n) {

@@ -103,9 +103,9 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
     }
     if (tid < ne) esdg_fx::fx_metric(fxe[tid], nscale + 3 * (size_t)(e0 + tid));
     esdg_cp_async_wait_all();  // these, and thread 0's edge elements of q
-    const bool ok = tile_wait(&bar, parity);
+    const bool ok = tile_wait(&bar, parity, a.timeout);
     if (__syncthreads_or(!ok)) {
-      if (tid == 0) atomicExch(&g_esdg_vol_timeout, 1);
+      if (tid == 0) atomicExch(a.timeout, 1);
       return;
     }
     // ---- prologue: node fields (FP64) and the elements' largest values ------------

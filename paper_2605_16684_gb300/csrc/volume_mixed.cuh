@@ -245,9 +245,9 @@ __global__ void __launch_bounds__(Mix<N, BG>::SH::THREADS, MixCfg<N, BG>::MINB)
       if (need_logs) pass(std::true_type{});
       else pass(std::false_type{});
     }
-    const bool landed = tile_wait(&bar, parity);
+    const bool landed = tile_wait(&bar, parity, a.timeout);
     if (__syncthreads_or(!landed)) {  // also: every sum written
-      if (tid == 0) atomicExch(&g_esdg_vol_timeout, 1);
+      if (tid == 0) atomicExch(a.timeout, 1);
       return;
     }
 

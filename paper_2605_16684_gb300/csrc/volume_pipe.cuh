@@ -8,26 +8,13 @@ namespace esdg_vol {
 // (member, first element) entries over member descriptors, which persistent CTAs walk
 // (TABLE: the batched server).  A tile's bulk copies complete on an mbarrier.
 #define ESDG_WAIT_LIMIT (1u << 18)  // polls; about 1 s on GB300
-// set when a bounded wait of a volume kernel ran out (one flag per
-// translation unit; read and cleared through es_dg_sync)
-static __device__ int g_esdg_vol_timeout;
-// 1 if it was set (and clears it), 0 if not, -1 on a CUDA error
-inline int take_timeout() {
-  int v = 0;
-  if (cudaMemcpyFromSymbol(&v, g_esdg_vol_timeout, sizeof(int)) != cudaSuccess) return -1;
-  if (v) {
-    const int z = 0;
-    if (cudaMemcpyToSymbol(g_esdg_vol_timeout, &z, sizeof(int)) != cudaSuccess) return -1;
-  }
-  return v ? 1 : 0;
-}
-// Wait for a tile's copies; false when the limit ran out, here or (looked at
-// every 1024 polls) in another CTA: the tiles after a failure do not each wait
-// out the limit.
-__device__ __forceinline__ bool tile_wait(unsigned long long* bar, unsigned parity) {
+// Wait for a tile's copies; false when the limit ran out, here or (flag, which the
+// caller sets, looked at every 1024 polls) in another CTA: the tiles after a failure do
+// not each wait out the limit.
+__device__ __forceinline__ bool tile_wait(unsigned long long* bar, unsigned parity, const int* flag) {
   for (unsigned it = 0; it < ESDG_WAIT_LIMIT; it += 1024u) {
     if (esdg_mbar_wait(bar, parity, 1024u)) return true;
-    if (*(volatile int*)&g_esdg_vol_timeout) break;
+    if (*(const volatile int*)flag) break;
   }
   return false;
 }
