@@ -41,8 +41,16 @@ struct F64 {
   static_assert(SH::NF == 18, "FP64 node fields");
 };
 
-template <int N, int MODE, bool TABLE>
-__global__ void __launch_bounds__(F64<N>::SH::THREADS, F64Cfg<N>::MINB)
+// ONE: the same kernel with the registers of a whole SM per CTA, for meshes of no more
+// tiles than SMs.  At N = 6 and 7 a lone CTA of 168 registers a thread leaves the pipes
+// waiting (N = 7, 4^3, one right-hand side, us, ONE against not: FP64 pairs at Mach 1 117
+// and 213, fixed point 46 and 62; with two CTAs an SM it is the slower one: 6^3 231 and
+// 220, 14^3 817 and 629 in fixed point); below, a tile has the registers it can use.
+template <int N>
+constexpr bool HAS_ONE = N >= 6;
+
+template <int N, int MODE, bool TABLE, bool ONE>
+__global__ void __launch_bounds__(F64<N>::SH::THREADS, ONE ? 1 : F64Cfg<N>::MINB)
     k_volume64(const __grid_constant__ EsdgMember one, const EsdgMember* __restrict__ members,
                const int2* __restrict__ tiles, const int* __restrict__ ntiles_d, int ntiles_1,
                const __grid_constant__ EsdgLGL L, double rkA, double rkB, unsigned phantom, int t1,
@@ -327,9 +335,10 @@ template <int N, int MODE>
 cudaError_t launch_volume64(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL& L,
                             const EsdgVolArgs& a, cudaStream_t s) {
   using SH = typename F64<N>::SH;
-  constexpr auto k = k_volume64<N, MODE, false>;
+  constexpr auto k = k_volume64<N, MODE, false, false>, one = k_volume64<N, MODE, false, HAS_ONE<N>>;
   const GridCap cap = pipe_grid_cap<k>(SH::THREADS, F64<N>::SMEM);
-  if (cap.ctas < 0) return cudaErrorInvalidConfiguration;
+  if (cap.ctas < 0 || pipe_grid_cap<one>(SH::THREADS, F64<N>::SMEM).ctas < 0)
+    return cudaErrorInvalidConfiguration;
   int ntiles, t1, s1;
   pipe_split(g.E, SH::EPB, cap.ctas, cap.sms / a.share, ntiles, t1, s1);
   if (ntiles == 0) return cudaSuccess;
@@ -337,7 +346,7 @@ cudaError_t launch_volume64(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL&
   // cost (path, clock) leave no SM waiting for the CTA with the costliest share, as a
   // persistent loop over a fixed share did (32^3 N = 4: 1.124 -> 0.976 ms; 16^3 N = 7:
   // 0.790 -> 0.763)
-  return esdg_launch(k, a.after, ntiles, SH::THREADS, F64<N>::SMEM, s, pipe_member(g, P, a), nullptr,
+  return esdg_launch(ntiles <= cap.sms / a.share ? one : k, a.after, ntiles, SH::THREADS, F64<N>::SMEM, s, pipe_member(g, P, a), nullptr,
                      nullptr, nullptr, ntiles, L, a.rkA, a.rkB, esdg_take_phantom(), t1, s1);
 }
 
@@ -346,7 +355,7 @@ template <int N>
 int batch_volume64(int what, const EsdgMember* members, const int2* tiles, const int* ntiles,
                    int grid, const EsdgLGL& L, double A, double B, cudaStream_t s) {
   using SH = typename F64<N>::SH;
-  constexpr auto k = k_volume64<N, 1, true>;
+  constexpr auto k = k_volume64<N, 1, true, false>;
   if (what == 1) return SH::EPB;
   if (what == 2) {
     int nb = 0;
