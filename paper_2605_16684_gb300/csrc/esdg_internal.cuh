@@ -308,10 +308,6 @@ __device__ __forceinline__ double esdg_f2d_pos(float f) {  // positive normal f
   const unsigned b = __float_as_uint(f);
   return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
 }
-__device__ __forceinline__ double esdg_A_t(double u) {
-  const float tail = fmaf(esdg_d2f_tail(u), 1.0f / 7.0f, 1.0f / 5.0f);
-  return fma(u, fma(u, esdg_f2d_pos(tail), 1.0 / 3.0), 1.0);
-}
 __device__ __forceinline__ double esdg_Q2_t(double u) {
   const float tail = fmaf(esdg_d2f_tail(u), 88.0f / 945.0f, 8.0f / 45.0f);  // -(u^2 coefficient tail)
   return fma(-u, fma(u, esdg_f2d_pos(tail), 2.0 / 3.0), 2.0);
@@ -412,18 +408,16 @@ struct EsdgMember {
 // Batched persistent launches over device work tables (tiles: int2 (member,
 // first element) for the volume, (member, first face node) in blocks of 256
 // for the faces; ntiles in device memory so the tables can change under a
-// captured graph).  variant selects the kernel (one at present).
+// captured graph).
 cudaError_t esdg_launch_face_batch(int N, int mixed, int bg, const EsdgMember* members,
                                    const int2* tiles, const int* ntiles, int grid, cudaStream_t s);
 // what: 0 launch (returns 0 or -1), 1 elements per tile, 2 CTAs per SM
-int esdg_volume_batch_f64(int what, int N, int variant, const EsdgMember* members, const int2* tiles,
+int esdg_volume_batch_f64(int what, int N, const EsdgMember* members, const int2* tiles,
                           const int* ntiles, int grid, const EsdgLGL& L, double A, double B,
                           cudaStream_t s);
-int esdg_volume_batch_mixed(int what, int N, int variant, const EsdgMember* members,
+int esdg_volume_batch_mixed(int what, int N, const EsdgMember* members,
                             const int2* tiles, const int* ntiles, int grid, const EsdgLGL& L,
                             double A, double B, cudaStream_t s);
-int esdg_volume_batch_variants_f64(int N);
-int esdg_volume_batch_variants_mixed(int N);
 
 // Test hook (es_dg_debug_inject_wait_timeout): bytes the next single-mesh
 // volume launch registers on its first barrier without copying them;

@@ -66,7 +66,7 @@ struct Member {
 
 struct Group {
   int N = 0, mixed = 0;
-  int variant = -1, grid_vol = 0, grid_face = 0;
+  int grid_vol = 0, grid_face = 0;  // grid_vol: CTAs of the volume launch, 0 until tuned
   EsdgLGL L{};
   int2* d_vt = nullptr;  // volume tiles
   int2* d_ft = nullptr;  // face tiles
@@ -128,8 +128,8 @@ struct es_dg_server {
   cudaGraphExec_t graph = nullptr;
   bool graph_valid = false;
   int use_graph = 1;
-  int force_variant = -1;  // ES_DG_BATCH_VARIANT: skip the autotuner (tests)
-  std::map<long long, std::pair<int, int>> tuned;  // (N, mixed) -> (variant, grid mult)
+  bool untuned = false;            // ES_DG_BATCH_VARIANT: skip the autotuner (tests)
+  std::map<long long, int> tuned;  // (N, mixed) -> CTAs per SM of the volume launch
   // statistics
   es_dg_server_stats_t st{};
   double t0 = 0;
@@ -151,18 +151,18 @@ int group_index(es_dg_server* s, int N, int mixed) {
   return -1;
 }
 
-int vol_epb(const Group& g, int variant) {
-  return g.mixed ? esdg_volume_batch_mixed(1, g.N, variant, nullptr, nullptr, nullptr, 0, g.L, 0, 0, 0)
-                 : esdg_volume_batch_f64(1, g.N, variant, nullptr, nullptr, nullptr, 0, g.L, 0, 0, 0);
+int vol_epb(const Group& g) {
+  return g.mixed ? esdg_volume_batch_mixed(1, g.N, nullptr, nullptr, nullptr, 0, g.L, 0, 0, 0)
+                 : esdg_volume_batch_f64(1, g.N, nullptr, nullptr, nullptr, 0, g.L, 0, 0, 0);
 }
-int vol_occ(const Group& g, int variant) {
-  return g.mixed ? esdg_volume_batch_mixed(2, g.N, variant, nullptr, nullptr, nullptr, 0, g.L, 0, 0, 0)
-                 : esdg_volume_batch_f64(2, g.N, variant, nullptr, nullptr, nullptr, 0, g.L, 0, 0, 0);
+int vol_occ(const Group& g) {
+  return g.mixed ? esdg_volume_batch_mixed(2, g.N, nullptr, nullptr, nullptr, 0, g.L, 0, 0, 0)
+                 : esdg_volume_batch_f64(2, g.N, nullptr, nullptr, nullptr, 0, g.L, 0, 0, 0);
 }
 int vol_launch(es_dg_server* s, const Group& g, double A, double B) {
-  const int r = g.mixed ? esdg_volume_batch_mixed(0, g.N, g.variant, s->d_members, g.d_vt, g.d_n,
+  const int r = g.mixed ? esdg_volume_batch_mixed(0, g.N, s->d_members, g.d_vt, g.d_n,
                                                   g.grid_vol, g.L, A, B, s->stream)
-                        : esdg_volume_batch_f64(0, g.N, g.variant, s->d_members, g.d_vt, g.d_n,
+                        : esdg_volume_batch_f64(0, g.N, s->d_members, g.d_vt, g.d_n,
                                                 g.grid_vol, g.L, A, B, s->stream);
   return r == 0 ? ES_DG_OK : cuda_fail(s, cudaGetLastError(), "volume batch launch");
 }
@@ -172,8 +172,8 @@ int face_launch(es_dg_server* s, const Group& g) {
   return e == cudaSuccess ? ES_DG_OK : cuda_fail(s, e, "face batch launch");
 }
 
-void build_tiles(es_dg_server* s, Group& g, int variant) {
-  const int epb = vol_epb(g, variant);
+void build_tiles(es_dg_server* s, Group& g) {
+  const int epb = vol_epb(g);
   g.vt.clear();
   g.ft.clear();
   for (size_t m = 0; m < s->active.size(); m++) {
@@ -247,18 +247,17 @@ int upload(es_dg_server* s) {
   return e == cudaSuccess ? ES_DG_OK : cuda_fail(s, e, "table upload sync");
 }
 
-// Autotune one group: every tile shape x grid multiplier, timed on the current
-// members with zero RK weights (B = 0 leaves the state unchanged; dq is
-// rewritten at the next stage 0 anyway).
-// tuning results shared by the servers of this process: (device, N, mixed) -> (variant, grid multiplier)
+// tuning results shared by the servers of this process: (device, N, mixed) -> CTAs per SM
 std::mutex g_tuned_mu;
-std::map<long long, std::pair<int, int>> g_tuned;
+std::map<long long, int> g_tuned;
 
+// Autotune one group: the grid of its volume launch, one or two rounds of resident CTAs,
+// timed on the current members with zero RK weights (B = 0 leaves the state unchanged; dq
+// is rewritten at the next stage 0 anyway).
 int autotune(es_dg_server* s, Group& g) {
-  const int nvar = g.mixed ? esdg_volume_batch_variants_mixed(g.N) : esdg_volume_batch_variants_f64(g.N);
-  if (s->force_variant >= 0) {
-    g.variant = s->force_variant < nvar ? s->force_variant : nvar - 1;
-    g.grid_vol = s->sms * vol_occ(g, g.variant);
+  const int occ = vol_occ(g);
+  if (s->untuned) {
+    g.grid_vol = s->sms * occ;
     s->graph_valid = false;
     return ES_DG_OK;
   }
@@ -271,48 +270,44 @@ int autotune(es_dg_server* s, Group& g) {
     if (jt != g_tuned.end()) it = s->tuned.insert({key, jt->second}).first;
   }
   if (it != s->tuned.end()) {
-    g.variant = it->second.first;
-    g.grid_vol = s->sms * it->second.second;
+    g.grid_vol = s->sms * it->second;
     return ES_DG_OK;
   }
+  build_tiles(s, g);
+  int st = upload(s);
+  if (st) return st;
+  // valid face fluxes for the volume launches being timed
+  if (face_launch(s, g)) return ES_DG_ECUDA;
   float best = 1e30f;
-  int bv = 0, bm = 1;
+  int per_sm = occ;
   cudaEvent_t a, b;
   cudaEventCreate(&a);
   cudaEventCreate(&b);
-  for (int v = 0; v < nvar; v++) {
-    build_tiles(s, g, v);
-    g.variant = v;
-    int st = upload(s);
-    if (st) return st;
-    // valid face fluxes for the volume launches being timed
-    if (face_launch(s, g)) return ES_DG_ECUDA;
-    const int occ = vol_occ(g, v);
-    for (int mult = 1; mult <= 2; mult++) {
-      g.grid_vol = s->sms * occ * mult;
-      if (vol_launch(s, g, 0.0, 0.0)) return ES_DG_ECUDA;  // warm-up
-      cudaEventRecord(a, s->stream);
-      for (int r = 0; r < 3; r++)
-        if (vol_launch(s, g, 0.0, 0.0)) return ES_DG_ECUDA;
-      cudaEventRecord(b, s->stream);
-      if (cudaEventSynchronize(b) != cudaSuccess) return ES_DG_ECUDA;
-      float ms = 0;
-      cudaEventElapsedTime(&ms, a, b);
-      if (ms < best) {
-        best = ms;
-        bv = v;
-        bm = occ * mult;
-      }
+  for (int mult = 1; mult <= 2 && st == ES_DG_OK; mult++) {
+    g.grid_vol = s->sms * occ * mult;
+    st = vol_launch(s, g, 0.0, 0.0);  // warm-up
+    cudaEventRecord(a, s->stream);
+    for (int r = 0; r < 3 && st == ES_DG_OK; r++) st = vol_launch(s, g, 0.0, 0.0);
+    cudaEventRecord(b, s->stream);
+    if (cudaEventSynchronize(b) != cudaSuccess) st = ES_DG_ECUDA;
+    float ms = 0;
+    cudaEventElapsedTime(&ms, a, b);
+    if (ms < best) {
+      best = ms;
+      per_sm = occ * mult;
     }
   }
   cudaEventDestroy(a);
   cudaEventDestroy(b);
-  g.variant = bv;
-  g.grid_vol = s->sms * bm;
-  s->tuned[key] = {bv, bm};
+  if (st) {
+    g.grid_vol = 0;
+    return ES_DG_ECUDA;
+  }
+  g.grid_vol = s->sms * per_sm;
+  s->tuned[key] = per_sm;
   {
     std::lock_guard<std::mutex> lk(g_tuned_mu);
-    g_tuned[gkey] = {bv, bm};
+    g_tuned[gkey] = per_sm;
   }
   s->graph_valid = false;
   return ES_DG_OK;
@@ -356,7 +351,7 @@ int rebuild(es_dg_server* s) {
     s->graph_valid = false;
   }
   for (Group& g : s->groups) {
-    if (g.variant < 0) {
+    if (!g.grid_vol) {
       // first time: tune on the members present (tables are built inside)
       bool any = false;
       for (auto& m : s->active) any |= (m->N == g.N && m->mixed == g.mixed);
@@ -364,11 +359,10 @@ int rebuild(es_dg_server* s) {
         int st = autotune(s, g);
         if (st) return st;
       } else {
-        g.variant = 0;
         g.grid_vol = s->sms;
       }
     }
-    build_tiles(s, g, g.variant);
+    build_tiles(s, g);
   }
   return upload(s);
 }
@@ -689,7 +683,7 @@ int es_dg_server_create(size_t hbm_budget_bytes, int max_slots, void* cuda_strea
   const char* g = std::getenv("ES_DG_NO_GRAPH");
   s->use_graph = !(g && g[0] == '1');
   const char* v = std::getenv("ES_DG_BATCH_VARIANT");
-  if (v && v[0] >= '0' && v[0] <= '9') s->force_variant = v[0] - '0';
+  s->untuned = v && v[0] >= '0' && v[0] <= '9';
   s->t0 = now_s();
   s->worker = std::thread(worker, s);
   *out = s;

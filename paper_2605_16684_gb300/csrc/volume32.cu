@@ -13,13 +13,10 @@ cudaError_t esdg_launch_volume_mixed(const EsdgGrid& g, const EsdgLGL& L, const 
   });
 }
 
-int esdg_volume_batch_variants_mixed(int) { return 1; }
-
 // what: 0 launch (returns 0 / -1), 1 elements per tile, 2 CTAs per SM
-int esdg_volume_batch_mixed(int what, int N, int variant, const EsdgMember* members,
+int esdg_volume_batch_mixed(int what, int N, const EsdgMember* members,
                           const int2* tiles, const int* ntiles, int grid, const EsdgLGL& L,
                           double A, double B, cudaStream_t s) {
-  if (variant != 0) return -1;
   return esdg_vol::for_order(N, -1, [&](auto n) {
     return esdg_vol::batch_volume32<n.value>(what, members, tiles, ntiles, grid, L, A, B, s);
   });

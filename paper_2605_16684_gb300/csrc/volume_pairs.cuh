@@ -24,12 +24,9 @@ struct Shape {
   // node fields: rq=rho/4, bh=b/2, ib=1/b, uh=u/2 (3), ph=phi/2, [lr, lb], nh=Ja/2 (9),
   // [background: rq'=rho'/4, bh'=b'/2, rq_bg, bh_bg, 1/b_bg, p_bg, p'=p-p_bg,
   //  moving background: u'/2 = (u - u_bg)/2 (3)]
-  static constexpr int F_LR = 7, F_LB = 8;
   static constexpr int F_NH = MIXED ? 7 : 9;
   static constexpr int F_BG = F_NH + 9;
   static constexpr int NF = F_NH + 9 + (BG ? 7 : 0) + (BG == 2 ? 3 : 0);
-  using R = typename std::conditional<MIXED, float, double>::type;
-  static constexpr size_t SMEM = sizeof(R) * (size_t)NF * NP * EPB;
 };
 
 template <typename R>
@@ -81,7 +78,7 @@ __device__ __forceinline__ Node<R> load_node(const R* __restrict__ S, int n, int
 // The artanh series of 1/<b>_log scaled by ce = 1/(2(gamma - 1)): the energy
 // flux only needs ce/<b>_log, so ce goes into the coefficients (computed once
 // per thread) and one FMA per pair folds the term into the energy bracket.
-// Tail beyond u^1 in FP32 (see esdg_A_t).
+// Tail beyond u^1 in FP32 (see esdg_d2f_tail).
 struct CeSeries {
   double c0, c1;    // ce, ce/3
   float c2f, c3f;   // ce/5, ce/7
