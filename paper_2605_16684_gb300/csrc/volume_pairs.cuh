@@ -5,6 +5,7 @@
 // Used by the FP64 kernel (volume_fp64.cuh) and the mixed one (volume_mixed.cuh),
 // single meshes and batches alike, so both give bitwise the same results.
 #pragma once
+#include <atomic>
 #include <cstring>
 #include <type_traits>
 
@@ -730,19 +731,21 @@ struct GridCap {
 template <auto k>
 GridCap pipe_grid_cap(int threads, size_t smem) {
   constexpr int MAXDEV = 64;
-  static GridCap cap[MAXDEV];
+  static std::atomic<unsigned long long> cap[MAXDEV];  // ctas 2^32 + sms, 0 until found
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAXDEV) return GridCap{-1, 0};
-  if (cap[dev].ctas == 0) {
+  unsigned long long c = cap[dev].load();
+  if (c == 0) {
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return GridCap{-1, 0};
     int per_sm = 0, nsm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || per_sm < 1)
       return GridCap{-1, 0};
-    cap[dev] = GridCap{per_sm * nsm, nsm};
+    c = (unsigned long long)(per_sm * nsm) << 32 | (unsigned)nsm;
+    cap[dev].store(c);
   }
-  return cap[dev];
+  return GridCap{(int)(c >> 32), (int)(unsigned)c};
 }
 
 // Tiles of a single mesh of E elements on a device that holds cap CTAs: full rounds
