@@ -304,15 +304,10 @@ __global__ void __launch_bounds__(Mix<N, BG>::SH::THREADS, MixCfg<N, BG>::MINB)
         double r[5];
 #pragma unroll
         for (int v = 0; v < 5; v++) {
-          // the background's own right-hand side: at rest (momentum only) in FP32, at
-          // N = 7 and for a moving one in FP64
-          if constexpr (BG == 1 && N < 7) {
-            r[v] = esdg_f2d(r32[v] + (v >= 1 && v <= 3 ? o.rb[v - 1] : 0.0f));
-          } else {
-            r[v] = esdg_f2d(r32[v]);
-            if (BG == 1 && v >= 1 && v <= 3) r[v] += o.rb[v - 1];
-            if (BG == 2) r[v] += o.rb[v];
-          }
+          // plus the background's own right-hand side (at rest: momentum only)
+          r[v] = esdg_f2d(r32[v]);
+          if (BG == 1 && v >= 1 && v <= 3) r[v] += o.rb[v - 1];
+          if (BG == 2) r[v] += o.rb[v];
         }
         if (rotating) {
           const double f = P.f0 + P.beta * (o.y - P.y0);
