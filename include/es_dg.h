@@ -405,11 +405,10 @@ void es_dg_server_destroy(es_dg_server* s);
  * for 3 doubles, written asynchronously on cuda_stream (a cudaStream_t, NULL =
  * legacy default stream); synchronise the stream before reading it.
  *
- * Scratch: the per-element partial sums live in a static device array sized
- * for ES_DG_NOALLOC_MAX_ELEMS elements (3 doubles each, 6 MiB), present on
+ * Scratch: the partial sums live in a static device array (29 KiB), present on
  * every GPU that loads the library until the process exits.  Meshes with more
- * elements, and physics that es_dg_create would reject (gamma <= 1, R <= 0,
- * p0 <= 0), get -ES_DG_EINVAL before any CUDA call.  Each call made while
+ * than ES_DG_NOALLOC_MAX_ELEMS elements, and physics that es_dg_create would
+ * reject (gamma <= 1, R <= 0, p0 <= 0), get -ES_DG_EINVAL before any CUDA call.  Each call made while
  * cuda_stream is not capturing looks up the array's device address
  * (cudaGetSymbolAddress) with the current device, so a device reset, which may
  * move the array, is picked up; a call made during a capture reuses the

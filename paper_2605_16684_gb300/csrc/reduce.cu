@@ -262,8 +262,8 @@ cudaError_t esdg_launch_integrals(const EsdgGrid& g, const EsdgLGL& L, const Esd
 // Some callers cannot allocate device memory at all: code running under a
 // memory pool it does not own, inside a framework that forbids cudaMalloc on
 // its hot path, or in a process whose allocator is already exhausted.  For
-// them the per-element partial sums live in the file-scope array below instead
-// of a handle's scratch buffer.  The array is created with the module on every
+// them the partial sums (one triple per CTA) live in the file-scope array below
+// instead of a handle's scratch buffer.  The array is created with the module on every
 // device that loads this library and stays there until the process exits.
 // ---------------------------------------------------------------------------
 #include <mutex>
@@ -272,7 +272,7 @@ cudaError_t esdg_launch_integrals(const EsdgGrid& g, const EsdgLGL& L, const Esd
 
 namespace {
 
-static __device__ __align__(256) double g_noalloc_partials[3 * ES_DG_NOALLOC_MAX_ELEMS];
+static __device__ __align__(256) double g_noalloc_partials[3 * SUM_CTAS];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_noalloc_mutex;
@@ -316,7 +316,7 @@ extern "C" int es_dg_integrals_noalloc(const es_dg_mesh* mesh, int N, const es_d
   if (!mesh || !q || !J || !x || !out3 || N < 1 || N > 7) return ES_DG_EINVAL;
   if (mesh->kx < 1 || mesh->ky < 1 || mesh->kz < 1) return ES_DG_EINVAL;
   const long long E = (long long)mesh->kx * mesh->ky * mesh->kz;
-  if (E > ES_DG_NOALLOC_MAX_ELEMS) return ES_DG_EINVAL;  // beyond the static scratch
+  if (E > ES_DG_NOALLOC_MAX_ELEMS) return ES_DG_EINVAL;  // the documented limit
   EsdgGrid g{};
   g.K[0] = mesh->kx;
   g.K[1] = mesh->ky;
@@ -345,8 +345,8 @@ extern "C" int es_dg_integrals_noalloc(const es_dg_mesh* mesh, int N, const es_d
   double* scratch = nullptr;
   int st = noalloc_scratch((cudaStream_t)cuda_stream, &scratch);
   if (st) return st;
-  // every partial the fold reads (the first E triples) is written by this
-  // call, so nothing needs clearing between calls
+  // every partial the fold reads (one triple per CTA) is written by this call,
+  // so nothing needs clearing between calls
   cudaError_t e = esdg_launch_integrals(g, L, P, q, J, x, scratch, out3, (cudaStream_t)cuda_stream);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? ES_DG_ENOMEM : ES_DG_ECUDA;
   return ES_DG_OK;
