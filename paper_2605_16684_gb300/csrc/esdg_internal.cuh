@@ -436,7 +436,7 @@ inline cudaError_t esdg_launch_volume(const EsdgGrid& g, const EsdgLGL& L, const
 #endif
 // Reductions with a scratch buffer of at least esdg_reduce_scratch(g) doubles;
 // the result lands in out[0] (CFL: the largest reference-space signal speed, 0
-// if no node has one) or out[0..2] (integrals: mass, energy, entropy), device memory.
+// if no node has one; out[1] is overwritten) or out[0..2] (integrals: mass, energy, entropy), device memory.
 size_t esdg_reduce_scratch(const EsdgGrid& g);
 cudaError_t esdg_launch_cfl(const EsdgGrid& g, const EsdgPhys& P, const double* q, const double* x,
                             const double* J, const double* Ja, double* scratch, double* out,

@@ -228,11 +228,11 @@ size_t esdg_reduce_scratch(const EsdgGrid& g) { return (size_t)g.E * 3; }
 cudaError_t esdg_launch_cfl(const EsdgGrid& g, const EsdgPhys& P, const double* q, const double* x,
                             const double* J, const double* Ja, double* scratch, double* out,
                             cudaStream_t s) {
-  // scratch: lambda per element in FP32, then its largest value
+  // scratch: lambda per element in FP32; its largest value behind the result, so that
+  // one memset clears both
   float* lam32 = reinterpret_cast<float*>(scratch);
-  unsigned* top = reinterpret_cast<unsigned*>(scratch + g.E);
-  cudaError_t err = cudaMemsetAsync(top, 0, sizeof(unsigned), s);
-  if (err == cudaSuccess) err = cudaMemsetAsync(out, 0, sizeof(double), s);
+  unsigned* top = reinterpret_cast<unsigned*>(out + 1);
+  cudaError_t err = cudaMemsetAsync(out, 0, 2 * sizeof(double), s);
   if (err != cudaSuccess) return err;
   const int warps = 8, most = SUM_CTAS;
   const int screen = (g.E + warps - 1) / warps;
