@@ -201,6 +201,7 @@ EsdgVolArgs vol_args(es_dg_t* h, const double* q_in, double* rhs_out) {
   a.status = h->status;
   a.timeout = h->timeout;
   a.share = 1;
+  a.early = 0;
   a.after = 0;
   return a;
 }

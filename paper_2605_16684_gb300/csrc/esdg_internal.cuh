@@ -172,14 +172,21 @@ __device__ __forceinline__ double esdg_ldexp(double x, int k) {
 // ---- launches that start while the launch before them in the stream ends
 // Device: wait until that launch is complete and its writes are visible.  First in
 // every kernel that esdg_launch starts, before any access to memory; without `after`
-// it is a no-op.  No kernel lets the next launch start before its own CTAs have ended
-// (griddepcontrol.launch_dependents): CTAs of the next launch that are placed while this
-// one's hold the SMs pile up on some of them, and a launch of up to a few CTAs per SM
-// waits for the fullest.  One LSRK step, us: started early / as here / plain launches:
-// mixed 4^3 N = 7 180 / 108 / 134, 8^3 N = 4 98 / 73 / 93; FP64 4^3 N = 3 127 / 128 / 151,
-// 6^3 N = 5 361 / 260 / 287, 8^3 N = 4 363 / 270 / 288; from 10^3 N = 6 on alike.
+// it is a no-op.
 __device__ __forceinline__ void esdg_wait_before() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Device: let the launch after this one start in the same way before this one's CTAs
+// have ended.  Kernels do without: CTAs of the next launch that are placed while this
+// one's hold the SMs pile up on some of them, and a launch of up to a few CTAs per SM
+// waits for the fullest.  One LSRK step, us: started early / not / plain launches: mixed
+// 4^3 N = 7 180 / 108 / 134, 8^3 N = 4 98 / 73 / 93; FP64 6^3 N = 5 361 / 260 / 287, 8^3
+// N = 4 363 / 270 / 288; from 10^3 N = 6 on within 1 %.  The exceptions
+// (EsdgVolArgs::early) are FP64 volume launches that leave half of the SMs idle, where the
+// interface kernel's CTAs find room (4^3 N = 3 117 against 119 us), and those of many
+// rounds of tiles, whose last round leaves room bit by bit (12^3 N = 7 2249 and 2271 us).
+__device__ __forceinline__ void esdg_start_next() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 // Host: launch k; after != 0 only when the launch before it in the stream is one of
 // this library's that calls esdg_wait_before (the stages of a step): it is then set up
@@ -389,6 +396,7 @@ struct EsdgVolArgs {
                          // density is not positive (null: not checked)
   int* timeout;          // set to 1 when a bounded wait of the kernel ran out (one word per device)
   int share;             // launches of this kind that run side by side (slabs of one mesh)
+  int early;             // lets the launch after it start before its own CTAs have ended
   int after;             // the launch before this one in the stream is the stage's interface kernel
 };
 // The mixed volume kernel without a background or with a moving one (its own

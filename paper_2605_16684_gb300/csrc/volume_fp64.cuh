@@ -69,7 +69,10 @@ __global__ void __launch_bounds__(F64<N>::SH::THREADS, ONE ? 1 : F64Cfg<N>::MINB
   double* const sm = reinterpret_cast<double*>(smraw) + F64<N>::S0;
   double* const xs = reinterpret_cast<double*>(smraw) + F64<N>::X0;
   const int tid = threadIdx.x;
-  if constexpr (!TABLE) esdg_wait_before();
+  if constexpr (!TABLE) {
+    esdg_wait_before();
+    if (one.a.early) esdg_start_next();
+  }
   const int ntiles = TABLE ? *ntiles_d : ntiles_1;
   if (tid == 0) {
     esdg_mbar_init(&bar, 1);
@@ -342,12 +345,15 @@ cudaError_t launch_volume64(const EsdgGrid& g, const EsdgPhys& P, const EsdgLGL&
   int ntiles, t1, s1;
   pipe_split(g.E, SH::EPB, cap.ctas, cap.sms / a.share, ntiles, t1, s1);
   if (ntiles == 0) return cudaSuccess;
+  EsdgMember m = pipe_member(g, P, a);
+  m.a.early = a.share == 1 && (2 * ntiles <= cap.sms || ntiles >= 4 * cap.ctas);
   // one CTA per tile: the hardware hands tiles out as CTAs end, so tiles of unequal
   // cost (path, clock) leave no SM waiting for the CTA with the costliest share, as a
   // persistent loop over a fixed share did (32^3 N = 4: 1.124 -> 0.976 ms; 16^3 N = 7:
   // 0.790 -> 0.763)
-  return esdg_launch(ntiles <= cap.sms / a.share ? one : k, a.after, ntiles, SH::THREADS, F64<N>::SMEM, s, pipe_member(g, P, a), nullptr,
-                     nullptr, nullptr, ntiles, L, a.rkA, a.rkB, esdg_take_phantom(), t1, s1);
+  return esdg_launch(ntiles <= cap.sms / a.share ? one : k, a.after, ntiles, SH::THREADS,
+                     F64<N>::SMEM, s, m, nullptr, nullptr, nullptr, ntiles, L, a.rkA, a.rkB,
+                     esdg_take_phantom(), t1, s1);
 }
 
 // batched (TABLE) launches; what: 0 launch (0 / -1), 1 elements per tile, 2 CTAs per SM
