@@ -145,7 +145,7 @@ __global__ void k_geometry(EsdgGrid g, EsdgLGL L, EsdgPhys P, double* __restrict
     const double* a = vg + (size_t)(k / np) * 3 * np + k % np;
     double v = 0.0;
     for (int c = 0; c < 3; c++) {
-      const double t = ldexp(a[c * np], -stretch[c]);
+      const double t = a[c * np] * __hiloint2double((1023 - max(stretch[c], -100)) << 20, 0);
       v += t * t;
     }
     hi = max(hi, mag(v));
