@@ -69,10 +69,10 @@ def mixed_volume_bytes_per_node(N):
     nq = N + 1
     return 2 * 40 + 2 * 20 + 11 * 4 + (3 * 8 + 4 * 4) + 3 * 4 + 6 * 5 * 4 * nq * nq / nq ** 3
 
-# DRAM traffic of one FP64 volume launch (k_volume64<4, 1, 0>): ncu capture of the same
-# kernel on the 24^3 case (dram__bytes_read.sum + dram__bytes_write.sum = 339.73 MB +
-# 103.75 MB for 13 824 elements), scaled to the 32^3 launch by the element count.
-VOLUME_FP64_TRAFFIC_BYTES = (339.73e6 + 103.75e6) * 32768 / 13824
+# DRAM traffic of one FP64 volume launch (k_volume64<4, 1, 0, 0>): ncu capture of the same
+# kernel on the 24^3 case (dram__bytes_read.sum + dram__bytes_write.sum = 339.50 MB +
+# 103.53 MB for 13 824 elements), scaled to the 32^3 launch by the element count.
+VOLUME_FP64_TRAFFIC_BYTES = (339.50e6 + 103.53e6) * 32768 / 13824
 
 # Vector issue rates of the part (per SM and clock): 2 FP64 FMA, 128 FP32 FMA.
 DFMA_PER_CLK_SM, FFMA_PER_CLK_SM = 2, 128

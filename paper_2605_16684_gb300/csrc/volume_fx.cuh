@@ -19,25 +19,28 @@
 // sum), and the pressure's scale stands above the energies' where they are much larger
 // (FxScale::dp): gamma near 1 and meshes far above z = 0 lost up to five bits of it.
 // Right-hand side without dissipation against long double, error over that of the FP64
-// pair by variable, N = 2 to 7: cubes at rest to 100 m/s 0.4 to 0.95, boxes of 1:1 to 1:1e5
-// 0.4 to 0.96, elements of 3 to 11 km 0.4 to 1.0, gamma 1.05 to 2 0.45 to 0.95; N = 1 up to
-// 1.1.
+// pair by variable, N = 2 to 7: cubes to 100 m/s 0.4 to 0.95, boxes of 1:1 to 1:1e5 0.4 to
+// 0.96, elements of 3 to 11 km 0.4 to 1.1, gamma 1.05 to 2 0.4 to 0.95, a mesh 10 to
+// 1000 km above z = 0 0.4 to 1.0; N = 1 up to 1.1.
 //
 // Whole kernel, before (FP64 pairs) and after, one launch: 32^3 N = 4 warped bubble
 // 3.400 -> 1.164 ms (narrow path), 16^3 N = 7 2.77 -> 0.79 ms, 16^3 N = 4 on a 2 km
 // box 0.494 -> 0.209 ms (wide path), 60 x 12 x 6 N = 4 channel 0.566 -> 0.233 ms
-// (tall path); with the launches of volume_fp64.cuh 0.973, 0.762 and 0.189 ms.
+// (tall path); with the launches of volume_fp64.cuh 0.966, 0.767 and 0.190 ms, and
+// 80 x 16 x 8 N = 4 channel 0.485 ms.
 //
 // Which elements take it (fx_path, fx_scales), decided per element so that a
 // result does not depend on the tile: all densities and 1/b = 2p/rho positive and
 // within 0.95 % (narrow) or 12 % (wide) of the first node's, or densities between
 // 0.21 and 1.12 of it (tall: a stratified element whose first node is its
-// lowest); metric terms in a sane range, gamma <= 2, velocities
-// up to about half the speed of sound.  An element whose internal energy or geopotential
-// difference is well above p/rho takes the tall path too, which gives the pressure a
-// scale of its own.  The lines lie where the correction series leave 2^-51 (narrow), 2^-55 (wide, tall); all other
+// lowest); metric terms in a sane range, gamma <= 2, velocities up to about 0.4 of the
+// speed of sound.  An element with stretched components, or whose energies stand well
+// above p/rho, takes the tall path too, the only one for any scales.  The lines lie
+// where the correction series leave 2^-51 (narrow), 2^-55 (wide, tall); all other
 // elements take pair64.  The wide path costs a pair about 900 cycles, the tall one
-// 1000.
+// 1050.  The coefficients of odd_poly and coth_poly are those of the polynomials in w = y^2
+// that interpolate (f(y)/y - 1)/w at the Chebyshev points of the path's interval, computed
+// in 50 digits and rounded to the scales they are used at.
 //
 // The pair is pair64's in a form that needs no reciprocal: with the node
 // fields x = ln(rho)/2, y = ln(b)/2 (relative to the element's first node) and
